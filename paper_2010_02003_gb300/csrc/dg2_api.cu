@@ -890,22 +890,18 @@ int dg2_get_state(dg2_ctx* c, double* planes, double* t) {
   if (r) return r;
   if (!planes) return fail(DG2_E_ARG, "planes is null");
   if (c->fp32) {
-    // FP32 free-surface modes -> FP64 depth modes h = eta - z
-    const int nx = c->f.nx, ny = c->f.ny;
-    const size_t n = (size_t)nx * ny;
-    std::vector<float> buf(10 * n);
-    for (int k = 0; k < 10; ++k)
-      CU(cudaMemcpy2DAsync(buf.data() + k * n, nx * sizeof(float), c->f.S + k * c->f.plane,
-                           c->f.pitch * sizeof(float), nx * sizeof(float), ny,
-                           cudaMemcpyDeviceToHost, c->st));
-    std::vector<float> z0, z1x, z1y;
-    if ((r = f32_topo_modes(c, z0, z1x, z1y))) return r;
-    for (size_t k = 0; k < n; ++k) {
-      planes[k] = ((double)buf[k] - (double)z0[k]) + (double)buf[9 * n + k];
-      planes[n + k] = (double)buf[n + k] - (double)z1x[k];
-      planes[2 * n + k] = (double)buf[2 * n + k] - (double)z1y[k];
+    // FP32 free-surface modes -> FP64 depth modes h = eta - z, formed on the device in
+    // the stage scratch T .. Q (free between steps) and copied out in dense runs of planes
+    const size_t n = (size_t)c->f.nx * c->f.ny;
+    const int room = (int)((c->lay.off_ZX - c->lay.off_T) / sizeof(double) / n);  // >= 8 planes
+    double* stage = (double*)(c->ws + c->lay.off_T);
+    for (int k = 0; k < 9; k += room) {
+      const int m = 9 - k < room ? 9 - k : room;
+      dg2::f32::state_out32_kernel<<<c->pgrid, c->pblock, 0, c->st>>>(c->f, stage, k, m);
+      if ((r = launch_check(c, 1))) return r;
+      CU(cudaMemcpyAsync(planes + (size_t)k * n, stage, (size_t)m * n * sizeof(double),
+                         cudaMemcpyDeviceToHost, c->st));
     }
-    for (size_t k = 3 * n; k < 9 * n; ++k) planes[k] = buf[k];
     Scalars s;
     if ((r = read_scalars(c, &s))) return r;
     if (t) *t = s.t;
@@ -925,37 +921,38 @@ int dg2_set_state(dg2_ctx* c, const double* planes, double t) {
   int r = check_arg_ctx(c, false);
   if (r) return r;
   if (!planes || !std::isfinite(t)) return fail(DG2_E_ARG, "bad planes or t");
-  const size_t n = (size_t)9 * c->d.nx * c->d.ny;
-  for (size_t k = 0; k < n; ++k)
-    if (!std::isfinite(planes[k])) return fail(DG2_E_ARG, "non-finite state value %zu", k);
+  // The planes go to scratch that is free between steps (T, and Q of an FP32 context) as
+  // dense FP64 runs; the device looks for non-finite values and, in FP32, converts them
+  // (h + z to the free-surface pair) into T.  The state S changes only once every value
+  // is known to be finite, so a refused call leaves it as it was.
+  const size_t n = (size_t)c->d.nx * c->d.ny;
+  unsigned long long* bad = (unsigned long long*)c->d.mpart;  // first non-finite value
+  CU(cudaMemsetAsync(bad, 0xff, sizeof *bad, c->st));
   if (c->fp32) {
-    // FP64 depth modes -> FP32 free-surface modes eta = h + z
-    const int nx = c->f.nx, ny = c->f.ny;
-    std::vector<float> z0, z1x, z1y;
-    if ((r = f32_topo_modes(c, z0, z1x, z1y))) return r;
-    std::vector<float> buf(10 * (size_t)nx * ny);
-    const size_t m = (size_t)nx * ny;
-    for (size_t k = 0; k < m; ++k) {
-      const double e0 = planes[k] + (double)z0[k];
-      buf[k] = (float)e0;
-      buf[9 * m + k] = (float)(e0 - (double)buf[k]);
-      buf[m + k] = (float)(planes[m + k] + (double)z1x[k]);
-      buf[2 * m + k] = (float)(planes[2 * m + k] + (double)z1y[k]);
+    double* stage = (double*)c->f.Q;  // 6 FP32 planes: three FP64 planes at a time
+    for (int k = 0; k < 9; k += 3) {
+      CU(cudaMemcpyAsync(stage, planes + (size_t)k * n, 3 * n * sizeof(double),
+                         cudaMemcpyHostToDevice, c->st));
+      dg2::f32::state_in32_kernel<<<c->pgrid, c->pblock, 0, c->st>>>(c->f, stage, k, bad);
     }
-    for (size_t k = 3 * m; k < 9 * m; ++k) buf[k] = (float)planes[k];
-    for (int k = 0; k < 10; ++k)
-      CU(cudaMemcpy2DAsync(c->f.S + k * c->f.plane, c->f.pitch * sizeof(float), buf.data() + k * m,
-                           nx * sizeof(float), nx * sizeof(float), ny, cudaMemcpyHostToDevice,
-                           c->st));
-    CU(cudaStreamSynchronize(c->st));
+    if ((r = launch_check(c, 3))) return r;
   } else {
-    const size_t w = (size_t)c->d.nx * sizeof(double), pb = (size_t)c->d.pitch * sizeof(double);
-    for (int k = 0; k < 9; ++k)
-      CU(cudaMemcpy2DAsync(c->d.S + k * c->d.plane, pb, planes + (size_t)k * c->d.nx * c->d.ny,
-                           w, w, c->d.ny, cudaMemcpyHostToDevice, c->st));
+    CU(cudaMemcpyAsync(c->d.T, planes, 9 * n * sizeof(double), cudaMemcpyHostToDevice, c->st));
+    dg2::state_check_kernel<<<c->pgrid, c->pblock, 0, c->st>>>(c->d, bad);
+    if ((r = launch_check(c, 1))) return r;
   }
+  unsigned long long first = 0;
+  CU(cudaMemcpyAsync(&first, bad, sizeof first, cudaMemcpyDeviceToHost, c->st));
   Scalars s;
   if ((r = read_scalars(c, &s))) return r;
+  if (first != ~0ull) return fail(DG2_E_ARG, "non-finite state value %llu", first);
+  if (c->fp32) {
+    CU(cudaMemcpyAsync(c->f.S, c->f.T, dg2::f32::kPlanes32 * (size_t)c->f.plane * sizeof(float),
+                       cudaMemcpyDeviceToDevice, c->st));
+  } else {
+    dg2::state_in_kernel<<<c->pgrid, c->pblock, 0, c->st>>>(c->d);
+    if ((r = launch_check(c, 1))) return r;
+  }
   s.t = t;
   s.done = 0;
   s.nonfinite = 0;
@@ -963,10 +960,12 @@ int dg2_set_state(dg2_ctx* c, const double* planes, double t) {
   s.t_end = INFINITY;
   s.next_sample = s.sample_every > 0.0 ? (std::floor(t / s.sample_every + 1e-9) + 1.0) * s.sample_every
                                        : INFINITY;
+  s.ledger_init = 1;  // the mass kernel below resets the ledger
   CU(cudaMemcpyAsync(c->d.sc, &s, sizeof s, cudaMemcpyHostToDevice, c->st));
   c->dem_set = 1;
   if ((r = reset_tiles(c))) return r;
-  if ((r = reset_ledger(c))) return r;
+  launch_mass(c);
+  if ((r = launch_check(c, 1))) return r;
   if ((r = recompute_dt(c))) return r;
   CU(cudaStreamSynchronize(c->st));
   return DG2_OK;

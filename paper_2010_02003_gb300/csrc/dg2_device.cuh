@@ -1574,6 +1574,30 @@ static __global__ void __launch_bounds__(kFinThreads) finalize_kernel(Dev d, int
   if (threadIdx.x == 0) open_lists(sc);
 }
 
+// Uploaded state (dg2_set_state): nine dense FP64 planes staged in T.  The check writes
+// the least index of a non-finite value to *bad (all ones: none); the copy takes the
+// planes to S.  Bound by HBM (72 bytes read, then 144 moved per cell) behind the upload;
+// the host loop over every value that it replaces took 9 ms for 2000 x 1000 cells, the
+// upload itself about 1 ms.
+static __global__ void __launch_bounds__(256) state_check_kernel(Dev d, unsigned long long* bad) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
+  if (i >= d.nx || j >= d.ny) return;
+  const long long n = (long long)d.nx * d.ny, c = (long long)j * d.nx + i;
+#pragma unroll
+  for (int k = 0; k < 9; ++k)
+    if (!isfinite(d.T[k * n + c])) {
+      atomicMin(bad, (unsigned long long)(k * n + c));
+      return;
+    }
+}
+static __global__ void __launch_bounds__(256) state_in_kernel(Dev d) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
+  if (i >= d.nx || j >= d.ny) return;
+  const long long n = (long long)d.nx * d.ny, c = (long long)j * d.nx + i;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) d.S[k * d.plane + (long long)j * d.pitch + i] = d.T[k * n + c];
+}
+
 // Courant reduction of the current state alone (after set-up or set_state).
 static __global__ void __launch_bounds__(256) rate_kernel(Dev d) {
   __shared__ double red[32];

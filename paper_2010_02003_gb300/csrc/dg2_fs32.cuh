@@ -505,6 +505,72 @@ static __device__ void finalize32_body(const D32& d, int lists_only) {
   if (threadIdx.x == 0) open_lists(sc);
 }
 
+// State in and out of an FP32 context (dg2_set_state, dg2_get_state): FP64 depth modes on
+// the host side, free-surface modes h + z here.  The conversions used to run in host loops
+// (25 ms in and 11 ms out for 2000 x 1000 cells); on the device they hide behind the copies
+// of the FP64 planes.  FP32 roundings keep denormals (the build flushes them elsewhere), so
+// a state goes through unchanged.
+__device__ __forceinline__ float to_f32(double x) {
+  float r;
+  asm("cvt.rn.f32.f64 %0, %1;" : "=f"(r) : "d"(x));
+  return r;
+}
+__device__ __forceinline__ float half_sum(float a, float b) {
+  float r;
+  asm("{\n.reg .f32 s;\nadd.rn.f32 s, %1, %2;\nmul.rn.f32 %0, s, 0f3f000000;\n}" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ double to_f64(float x) {
+  double r;
+  asm("cvt.f64.f32 %0, %1;" : "=d"(r) : "f"(x));
+  return r;
+}
+
+// The bed mode of a cell that depth plane k (0 average, 1 x slope, 2 y slope) stands on.
+__device__ __forceinline__ double bed_mode(const D32& d, int i, int j, int k) {
+  const float* z = k == 2 ? d.ZY + (long long)j * d.pitch + i : d.ZX + (long long)j * d.zpx + i;
+  const float lo = z[0], hi = k == 2 ? z[d.pitch] : z[1];
+  return to_f64(half_sum(hi, k == 0 ? lo : -lo));
+}
+
+// Planes k0 .. k0 + 2 of an uploaded state, dense in `in`, into T (eta0's remainder with
+// plane 0); *bad takes the least index of a non-finite value (all ones: none).
+static __global__ void __launch_bounds__(256) state_in32_kernel(D32 d, const double* __restrict__ in,
+                                                                int k0, unsigned long long* bad) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
+  if (i >= d.nx || j >= d.ny) return;
+  const long long n = (long long)d.nx * d.ny, c = (long long)j * d.nx + i;
+  const long long P = d.plane, o = (long long)j * d.pitch + i;
+  for (int q = 0; q < 3; ++q) {
+    const int k = k0 + q;
+    double v = in[q * n + c];
+    if (!isfinite(v)) {
+      atomicMin(bad, (unsigned long long)(k * n + c));
+      return;
+    }
+    if (k < 3) v = v + bed_mode(d, i, j, k);
+    const float f = to_f32(v);
+    d.T[k * P + o] = f;
+    if (k == 0) d.T[E0L * P + o] = to_f32(v - to_f64(f));
+  }
+}
+
+// Planes k0 .. k0 + m - 1 of the state as dense FP64 depth modes.
+static __global__ void __launch_bounds__(256) state_out32_kernel(D32 d, double* __restrict__ out,
+                                                                 int k0, int m) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
+  if (i >= d.nx || j >= d.ny) return;
+  const long long n = (long long)d.nx * d.ny, c = (long long)j * d.nx + i;
+  const long long P = d.plane, o = (long long)j * d.pitch + i;
+  for (int q = 0; q < m; ++q) {
+    const int k = k0 + q;
+    double v = to_f64(d.S[k * P + o]);
+    if (k < 3) v = v - bed_mode(d, i, j, k);
+    if (k == 0) v = v + to_f64(d.S[E0L * P + o]);
+    out[q * n + c] = v;
+  }
+}
+
 static __global__ void __launch_bounds__(256) rate32_kernel(D32 d) {
   __shared__ double red[32];
   __shared__ bool last;
