@@ -252,6 +252,21 @@ void mirror(dg2_ctx* c) {
   f.tiles = d.tiles;
 }
 
+// The FP64 DG2 stage kernel of a variant, stage and Riemann solver.
+using StageFn = void (*)(Dev);
+StageFn stage64(bool ll, int stage, bool roe) {
+  if (roe) {
+    if (ll) return stage == 1 ? dg2::stage_kernel<true, 1, true> : dg2::stage_kernel<true, 2, true>;
+    return stage == 1 ? dg2::stage_kernel<false, 1, true> : dg2::stage_kernel<false, 2, true>;
+  }
+  if (ll) return stage == 1 ? dg2::stage_kernel<true, 1, false> : dg2::stage_kernel<true, 2, false>;
+  return stage == 1 ? dg2::stage_kernel<false, 1, false> : dg2::stage_kernel<false, 2, false>;
+}
+void launch_stage64(dg2_ctx* c, bool ll, int stage) {
+  stage64(ll, stage, c->d.flux == DG2_ROE)<<<stage == 1 ? c->g_st1 : c->g_st2, c->sblock,
+                                             sizeof(dg2::StageSmem), c->st>>>(c->d);
+}
+
 // Enqueues one RK2 step: friction, stage 1, stage 2, finalize, lists (5 kernels; 4 in
 // FP32, whose stages apply friction themselves).  With `timed`, records an event before
 // and after each kernel.
@@ -290,15 +305,13 @@ void enqueue_step(dg2_ctx* c, bool timed = false) {
   if (c->fp32) {
     dg2::ens::launch_stage32(c->e1, tile_w(c), ll, 1, c->g_st1, c->st);
   } else {
-    if (ll) dg2::stage_kernel<true, 1><<<c->g_st1, c->sblock, sizeof(dg2::StageSmem), c->st>>>(d);
-    else dg2::stage_kernel<false, 1><<<c->g_st1, c->sblock, sizeof(dg2::StageSmem), c->st>>>(d);
+    launch_stage64(c, ll, 1);
   }
   if (e) cudaEventRecord(e[2], c->st);
   if (c->fp32) {
     dg2::ens::launch_stage32(c->e1, tile_w(c), ll, 2, c->g_st2, c->st);
   } else {
-    if (ll) dg2::stage_kernel<true, 2><<<c->g_st2, c->sblock, sizeof(dg2::StageSmem), c->st>>>(d);
-    else dg2::stage_kernel<false, 2><<<c->g_st2, c->sblock, sizeof(dg2::StageSmem), c->st>>>(d);
+    launch_stage64(c, ll, 2);
   }
   if (e) cudaEventRecord(e[3], c->st);
   launch_finalize(c, 0);
@@ -468,7 +481,9 @@ int dg2_init_grid(dg2_ctx** out, int nx, int ny, double dx, double dy, const dg2
   d.nx = nx; d.ny = ny; d.pitch = L.pitch; d.plane = L.plane;
   d.dx = dx; d.dy = dy; d.inv_dx = 1.0 / dx; d.inv_dy = 1.0 / dy;
   d.g = p.g; d.cfl = p.cfl; d.ds = p.ds_thresh; d.dt_max = p.dt_max;
-  d.tol = p.tol_dry == 0.0 ? 0.0 : p.tol_dry;  // +0: the bit-pattern comparisons want c >= +0
+  // Depths of 1e-300 m and less count as dry whatever the tolerance: 1 / h of a wet depth then
+  // has a normal argument (and the bit-pattern comparisons want c >= +0).
+  d.tol = p.tol_dry > 1e-300 ? p.tol_dry : 1e-300;
   for (int k = 0; k < 4; ++k) d.bc[k] = p.bc[k];
   c->fp32 = p.precision == DG2_FP32;
   // plane buffers: FP64 depth modes, or FP32 free-surface modes (the FP64
@@ -545,28 +560,11 @@ int dg2_init_grid(dg2_ctx** out, int nx, int ny, double dx, double dy, const dg2
     const bool ll = p.variant == DG2_LL, f32 = p.precision == DG2_FP32;
     int o1 = 1, o2 = 1;
     // the FP64 stage tile's shared memory is above the 48 KB static limit
-    cudaFuncSetAttribute(dg2::stage_kernel<true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sizeof(dg2::StageSmem));
-    cudaFuncSetAttribute(dg2::stage_kernel<true, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sizeof(dg2::StageSmem));
-    cudaFuncSetAttribute(dg2::stage_kernel<false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sizeof(dg2::StageSmem));
-    cudaFuncSetAttribute(dg2::stage_kernel<false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sizeof(dg2::StageSmem));
+    for (int k = 0; k < 8; ++k)
+      cudaFuncSetAttribute(stage64(k & 1, 1 + (k >> 1 & 1), k >> 2),
+                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(dg2::StageSmem));
     if (f32) {
       dg2::ens::occupancy32(tile_w(c), ll, &o1, &o2);
-    } else {
-      if (ll) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, dg2::stage_kernel<true, 1>, dg2::TX * dg2::TY,
-                                                      sizeof(dg2::StageSmem));
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o2, dg2::stage_kernel<true, 2>, dg2::TX * dg2::TY,
-                                                      sizeof(dg2::StageSmem));
-      } else {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, dg2::stage_kernel<false, 1>, dg2::TX * dg2::TY,
-                                                      sizeof(dg2::StageSmem));
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o2, dg2::stage_kernel<false, 2>, dg2::TX * dg2::TY,
-                                                      sizeof(dg2::StageSmem));
-      }
     }
     cudaGetLastError();
     const int nt = d.tiles.ntiles;
@@ -577,9 +575,8 @@ int dg2_init_grid(dg2_ctx** out, int nx, int ny, double dx, double dy, const dg2
     // as they free up); measured faster than a persistent grid looping over the
     // list (floodplain 2000 x 1000 from t = 1 h: 0.060 -> 0.051 ms per step)
     c->g_fric = nt;
-    const bool loop = f32 ? true : (p.scheme == DG2_SCHEME_DG2 && DG2_TILE_LOOP64);
-    c->g_st1 = loop ? gsz(o1) : nt;
-    c->g_st2 = loop ? gsz(o2) : nt;
+    c->g_st1 = f32 ? gsz(o1) : nt;
+    c->g_st2 = f32 ? gsz(o2) : nt;
   }
 
   // zero the state, topography and scalars; t_end / samples at +inf

@@ -226,76 +226,97 @@ __device__ __forceinline__ double min_nn(double a, double b) { return fbits(b) <
 __device__ __forceinline__ bool nonzero(double x) { return (fbits(x) << 1) != 0; }
 
 // ---------------------------------------------------------------------------
+// FP64 reciprocal and square root in few FP64 instructions
+// ---------------------------------------------------------------------------
+// The FP64 pipe bounds the stage kernels, and a compiled 1 / x or sqrt(x) is about
+// nine instructions on it with a branch to a slow path.  These start from the
+// hardware's 32-bit-mantissa-word approximations (PTX rcp.approx / rsqrt.approx)
+// and refine them: the reciprocal by one third-order Householder step
+// r (1 + e + e^2), e = 1 - x r (3 instructions); the root by two of Heron's steps
+// s + (x - s^2) y / 2 with the same y ~ x^(-1/2) (5 instructions), whose residuals
+// are exact to a rounding.  Over 2^28 arguments the relative residuals stay below
+// 1.01 x 2^-53 (the approximations': 1.0e-6 and 1.9e-6).
+__device__ __forceinline__ double rcp64(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  double e = fma(-x, r, 1.0);
+  e = fma(e, e, e);
+  return fma(r, e, r);
+}
+// x >= 0; 0 below the normal range
+__device__ __forceinline__ double sqrt64(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  // y / 2 by its exponent (y is normal for normal x)
+  const double h = __hiloint2double(__double2hiint(y) - 0x00100000, __double2loint(y));
+  const double t = x * y;
+  double s = fma(fma(-t, t, x), h, t);
+  s = fma(fma(-s, s, x), h, s);
+  return __double2hiint(x) < 0x00100000 ? 0.0 : s;
+}
+// x / 2, on the integer units unless the result is below the normal range
+__device__ __forceinline__ double half64(double x) {
+  const int hi = __double2hiint(x), e = hi & 0x7ff00000;
+  if (e <= 0x00100000) return nonzero(x) ? 0.5 * x : x;
+  return __hiloint2double(e == 0x7ff00000 ? hi : hi - 0x00100000, __double2loint(x));
+}
+
+// ---------------------------------------------------------------------------
 // Point-state helpers
 // ---------------------------------------------------------------------------
 
-// A revised face limit (Sec. 2.1.2): h* = max(0, h), velocities q/h above
-// tol_dry and zero otherwise, q* = h* u.  The velocities are kept for the flux.
-struct Lim {
-  double h, qx, qy, u, v;
+// A face flux in the face's frame: mass, normal momentum less the lower (left) side's
+// hydrostatic pressure g hL^2 / 2, tangential momentum, and dp = g (hL^2 - hR^2) / 2, so
+// that n + dp is the normal momentum less the upper (right) side's pressure.  A cell's own
+// pressures never enter the flux differences then: with its own revised face depths h and
+// beds z they regroup with the bed terms of Eqs. 4a-c into g / 2 (hE +- hW) times the
+// difference of the faces' free surfaces (hE + zE) - (hW + zW) (stage_tile), which takes
+// fewer operations, and no pressure of tens of units is left to cancel.
+struct Flux {
+  double h, n, t, dp;
 };
-
-struct F3 {
-  double h, x, y;
-};
-
-__device__ __forceinline__ Lim revise(double h, double qx, double qy, double tol) {
-  Lim r;
-  if (above(h, tol)) {
-    const double ih = 1.0 / h;
-    r.u = qx * ih;
-    r.v = qy * ih;
-  } else {
-    r.u = 0.0;
-    r.v = 0.0;
-  }
-  r.h = pos_part(h);
-  r.qx = r.h * r.u;
-  r.qy = r.h * r.v;
-  return r;
+__device__ __forceinline__ double pressure_step(double hL, double hR, double g) {
+  return (0.5 * g) * (hL - hR) * (hL + hR);
 }
 
 // HLL flux normal to a face (Toro's wave-speed estimates with the dry-bed
-// forms).  n = normal, t = tangential component; (un, ut) are the limit's
-// velocities.  Returns (mass, normal momentum, tangential momentum).
-__device__ __forceinline__ F3 hll(double hL, double qnL, double qtL, double unL, double utL,
-                                  double hR, double qnR, double qtR, double unR, double utR,
-                                  double g, double tol) {
-  F3 f;
-  const bool dL = !above(hL, tol), dR = !above(hR, tol);
-  if (dL && dR) {
-    f.h = 0.0; f.x = 0.0; f.y = 0.0;
+// forms).  n = normal, t = tangential component; (un, ut) are the limit's velocities.
+//
+// With the invariants I = uL + 2 cL and J = uR - 2 cR the two-rarefaction speeds
+// u* -+ c* are (I + 3 J) / 4 and (3 I + J) / 4, and the dry-bed speeds are I and J
+// themselves.  The speeds are clamped at 0 from either side, so one formula
+// F = FL + b (FR - FL) - b sR (UR - UL), b = -sL / (sR - sL), covers the supercritical
+// cases too (b is 0, or 1 to a rounding with sR = 0) without branches, and equal sides
+// give their flux exactly: 42 FP64 instructions, about 70 before.
+__device__ __forceinline__ Flux hll(double hL, double qnL, double qtL, double unL, double utL,
+                                    double hR, double qnR, double qtR, double unR, double utR,
+                                    double g, double tol) {
+  Flux f;
+  const bool wL = above(hL, tol), wR = above(hR, tol);
+  f.dp = pressure_step(hL, hR, g);
+  if (!wL && !wR) {
+    f.h = 0.0; f.n = -(0.5 * g * hL) * hL; f.t = 0.0;
     return f;
   }
-  const double cL = sqrt(g * hL), cR = sqrt(g * hR);
-  double sL, sR;
-  if (dL) {
-    sL = unR - 2.0 * cR;
-    sR = unR + cR;
-  } else if (dR) {
-    sL = unL - cL;
-    sR = unL + 2.0 * cL;
-  } else {
-    const double us = 0.5 * (unL + unR) + cL - cR;
-    const double cs = 0.5 * (cL + cR) + 0.25 * (unL - unR);
-    sL = min2(unL - cL, us - cs);
-    sR = max2(unR + cR, us + cs);
+  const double cL = sqrt64(g * hL), cR = sqrt64(g * hR);
+  const double A = unL - cL, B = unR + cR;
+  const double I = fma(2.0, cL, unL), J = fma(-2.0, cR, unR);
+  double sL = wL ? A : J, sR = wR ? B : I;
+  if (wL && wR) {
+    sL = min2(A, fma(0.75, J, 0.25 * I));
+    sR = max2(B, fma(0.75, I, 0.25 * J));
   }
-  // physical normal flux [h un, h un^2 + g h^2 / 2, h un ut] of each side
-  const double fLh = hL * unL, fLn = hL * unL * unL + 0.5 * g * hL * hL, fLt = hL * unL * utL;
-  const double fRh = hR * unR, fRn = hR * unR * unR + 0.5 * g * hR * hR, fRt = hR * unR * utR;
-  if (!is_neg(sL)) {
-    f.h = fLh; f.x = fLn; f.y = fLt;
-    return f;
-  }
-  if (!is_pos(sR)) {
-    f.h = fRh; f.x = fRn; f.y = fRt;
-    return f;
-  }
-  const double inv = 1.0 / (sR - sL), sLR = sL * sR;
-  f.h = (sR * fLh - sL * fRh + sLR * (hR - hL)) * inv;
-  f.x = (sR * fLn - sL * fRn + sLR * (qnR - qnL)) * inv;
-  f.y = (sR * fLt - sL * fRt + sLR * (qtR - qtL)) * inv;
+  sL = is_neg(sL) ? sL : 0.0;
+  sR = pos_part(sR);
+  // momentum fluxes [h un^2, h un ut] of each side, the right one with the pressure step;
+  // a dry side moves nothing
+  const double mL = wL ? qnL : 0.0, mR = wR ? qnR : 0.0;
+  const double b = -sL * rcp64(sR - sL), c = b * sR;
+  const double xL = mL * unL, xR = fma(mR, unR, -f.dp);
+  const double yL = mL * utL, yR = mR * utR;
+  f.h = fma(b, mR - mL, fma(c, hL - hR, mL));
+  f.n = fma(b, xR - xL, fma(c, qnL - qnR, xL));
+  f.t = fma(b, yR - yL, fma(c, qtL - qtR, yL));
   return f;
 }
 
@@ -314,12 +335,13 @@ __device__ __forceinline__ double harten(double lam, double lamL, double lamR) {
 // the physical fluxes minus the upwinding of the waves of the Roe-linearised
 // system (Roe averages, eigenvalues u^ -+ c^ and u^, wave strengths
 // (dh -+ h^ du / c^) / 2 and h^ dt), Harten's entropy fix on the acoustic waves.
-__device__ __forceinline__ F3 roe(double hL, double qnL, double qtL, double unL, double utL,
-                                  double hR, double qnR, double qtR, double unR, double utR,
-                                  double g, double tol) {
-  F3 f;
+__device__ __forceinline__ Flux roe(double hL, double qnL, double qtL, double unL, double utL,
+                                    double hR, double qnR, double qtR, double unR, double utR,
+                                    double g, double tol) {
+  Flux f;
+  f.dp = pressure_step(hL, hR, g);
   if (hL <= tol && hR <= tol) {
-    f.h = 0.0; f.x = 0.0; f.y = 0.0;
+    f.h = 0.0; f.n = -(0.5 * g * hL) * hL; f.t = 0.0;
     return f;
   }
   const double sL = sqrt(hL), sR = sqrt(hR);
@@ -335,65 +357,34 @@ __device__ __forceinline__ F3 roe(double hL, double qnL, double qtL, double unL,
   const double e1 = harten(l1, unL - cL, unR - cR), e2 = fabs(uh);
   const double e3 = harten(l3, unL + cL, unR + cR);
   const double w1 = e1 * a1, w2 = e2 * a2, w3 = e3 * a3;
-  const double fLh = hL * unL, fLn = hL * unL * unL + 0.5 * g * hL * hL, fLt = hL * unL * utL;
-  const double fRh = hR * unR, fRn = hR * unR * unR + 0.5 * g * hR * hR, fRt = hR * unR * utR;
+  // the physical fluxes less the left pressure
+  const double fLh = hL * unL, fLn = hL * unL * unL, fLt = hL * unL * utL;
+  const double fRh = hR * unR, fRn = hR * unR * unR - f.dp, fRt = hR * unR * utR;
   f.h = 0.5 * (fLh + fRh) - 0.5 * (w1 + w3);
-  f.x = 0.5 * (fLn + fRn) - 0.5 * (w1 * l1 + w3 * l3);
-  f.y = 0.5 * (fLt + fRt) - 0.5 * (w1 * vh + w2 + w3 * vh);
+  f.n = 0.5 * (fLn + fRn) - 0.5 * (w1 * l1 + w3 * l3);
+  f.t = 0.5 * (fLt + fRt) - 0.5 * (w1 * vh + w2 + w3 * vh);
   return f;
 }
 
-// x-face flux: returns [F^h, F^qx, F^qy].
-__device__ __forceinline__ F3 flux_x(const Lim& L, const Lim& R, double g, double tol,
-                                     int flux = 0) {
-  if (flux == 1) return roe(L.h, L.qx, L.qy, L.u, L.v, R.h, R.qx, R.qy, R.u, R.v, g, tol);
-  return hll(L.h, L.qx, L.qy, L.u, L.v, R.h, R.qx, R.qy, R.u, R.v, g, tol);
-}
-
-// y-face flux in the rotated frame, mapped back: returns [G^h, G^qx, G^qy].
-__device__ __forceinline__ F3 flux_y(const Lim& S, const Lim& N, double g, double tol,
-                                     int flux = 0) {
-  F3 r = flux == 1 ? roe(S.h, S.qy, S.qx, S.v, S.u, N.h, N.qy, N.qx, N.v, N.u, g, tol)
-                   : hll(S.h, S.qy, S.qx, S.v, S.u, N.h, N.qy, N.qx, N.v, N.u, g, tol);
-  F3 o;
-  o.h = r.h; o.x = r.y; o.y = r.x;
-  return o;
-}
-
-// Face flux along x or y by a run-time flag: the normal and tangential
-// components selected, so a warp holding both kinds of faces evaluates one flux
-// (the same arithmetic as flux_x / flux_y).
-__device__ __forceinline__ F3 flux_dir(const Lim& A, const Lim& B, bool ydir, double g, double tol,
-                                       int flux) {
-  const double an = ydir ? A.qy : A.qx, at = ydir ? A.qx : A.qy;
-  const double aun = ydir ? A.v : A.u, aut = ydir ? A.u : A.v;
-  const double bn = ydir ? B.qy : B.qx, bt = ydir ? B.qx : B.qy;
-  const double bun = ydir ? B.v : B.u, but = ydir ? B.u : B.v;
-  const F3 r = flux == 1 ? roe(A.h, an, at, aun, aut, B.h, bn, bt, bun, but, g, tol)
-                         : hll(A.h, an, at, aun, aut, B.h, bn, bt, bun, but, g, tol);
-  F3 o;
-  o.h = r.h;
-  o.x = ydir ? r.y : r.x;
-  o.y = ydir ? r.x : r.y;
-  return o;
-}
-
-// Physical flux F (x) or G (y) of a point state, velocities by the tol rule.
-__device__ __forceinline__ F3 phys_flux(double h, double qx, double qy, double g, double tol,
-                                        bool ydir) {
-  double u = 0.0, v = 0.0;
-  if (above(h, tol)) {
-    const double ih = 1.0 / h;
-    u = qx * ih;
-    v = qy * ih;
-  }
+// Pressure-free physical fluxes (mass q, normal momentum q u, tangential momentum) of a
+// direction's two Gauss points, summed and doubled, velocities by the tol rule.  (hs, ns,
+// ts) are the sums of the cell's two face states along it, (hd, nd, td) their differences
+// (the dummy modes of Eq. 5, doubled): the points are (s +- d / sqrt(3)) / 2, kept doubled.
+struct F3 {
+  double h, n, t;
+};
+__device__ __forceinline__ F3 gauss_pair(double hs, double ns, double ts, double hd, double nd,
+                                         double td, double tol2) {
+  const double r3 = 0.57735026918962576;
+  const double h1 = fma(r3, hd, hs), h2 = fma(-r3, hd, hs);
+  const double n1 = fma(r3, nd, ns), n2 = fma(-r3, nd, ns);
+  const double t1 = fma(r3, td, ts), t2 = fma(-r3, td, ts);
+  const bool w1 = above(h1, tol2), w2 = above(h2, tol2);
+  const double u1 = w1 ? n1 * rcp64(h1) : 0.0, u2 = w2 ? n2 * rcp64(h2) : 0.0;
   F3 f;
-  const double p = 0.5 * g * h * h;
-  if (!ydir) {
-    f.h = h * u; f.x = h * u * u + p; f.y = h * u * v;
-  } else {
-    f.h = h * v; f.x = h * u * v; f.y = h * v * v + p;
-  }
+  f.h = (w1 ? n1 : 0.0) + (w2 ? n2 : 0.0);
+  f.n = fma(n1, u1, n2 * u2);
+  f.t = fma(t1, u1, t2 * u2);
   return f;
 }
 
@@ -522,17 +513,16 @@ __device__ __forceinline__ void wetdry(double* m, double z0, double z1x, double 
     for (int k = 1; k < 9; ++k) m[k] = 0.0;
     return;
   }
-  const double eta0 = h0 + z0;
-  // x direction
-  {
-    const bool fe = !above(h0 + m[H1X], tol) && !gt(z0 + z1x, eta0);
-    const bool fw = !above(h0 - m[H1X], tol) && !gt(z0 - z1x, eta0);
-    if (fe || fw) { m[H1X] = 0.0; m[QX1X] = 0.0; m[QY1X] = 0.0; }
-  }
-  {
-    const bool fn = !above(h0 + m[H1Y], tol) && !gt(z0 + z1y, eta0);
-    const bool fs = !above(h0 - m[H1Y], tol) && !gt(z0 - z1y, eta0);
-    if (fn || fs) { m[H1Y] = 0.0; m[QX1Y] = 0.0; m[QY1Y] = 0.0; }
+  const bool de = !above(h0 + m[H1X], tol), dw = !above(h0 - m[H1X], tol);
+  const bool dn = !above(h0 + m[H1Y], tol), ds = !above(h0 - m[H1Y], tol);
+  if (de || dw || dn || ds) {
+    const double eta0 = h0 + z0;
+    if ((de && !gt(z0 + z1x, eta0)) || (dw && !gt(z0 - z1x, eta0))) {
+      m[H1X] = 0.0; m[QX1X] = 0.0; m[QY1X] = 0.0;
+    }
+    if ((dn && !gt(z0 + z1y, eta0)) || (ds && !gt(z0 - z1y, eta0))) {
+      m[H1Y] = 0.0; m[QX1Y] = 0.0; m[QY1Y] = 0.0;
+    }
   }
 }
 
@@ -597,8 +587,8 @@ __device__ __forceinline__ float block_max_f(float v, float* sh) {
 // Courant wave-speed rate of a cell: max((|u|+c)/dx, (|v|+c)/dy) if wet.
 __device__ __forceinline__ double cell_rate(const Dev& d, double h0, double qx0, double qy0) {
   if (!above(h0, d.tol)) return 0.0;
-  const double ih = 1.0 / h0;
-  const double u = qx0 * ih, v = qy0 * ih, c = sqrt(d.g * h0);
+  const double ih = rcp64(h0);
+  const double u = qx0 * ih, v = qy0 * ih, c = sqrt64(d.g * h0);
   return max_nn((fabs(u) + c) * d.inv_dx, (fabs(v) + c) * d.inv_dy);
 }
 
@@ -672,30 +662,28 @@ static __global__ void init_kernel(Dev d, const double* __restrict__ zc, const d
 }
 
 // Point-implicit friction (Sec. 2.1.3) at one point: q /= 1 + dt g n^2 |q| / h^(7/3).
-// h^(-7/3) for h in (1e-30, 1e30): the inverse cube root r = h^(-1/3) by two
-// Newton steps on f(r) = r^-3 - h, r <- r + r (1 - h r^3) / 3 (the error
-// squares at each step), from the FP32 inverse cube root as the seed (relative
-// error ~1e-7, so the second step reaches FP64 rounding), then r^7 = r (r^3)^2:
-// no FP64 cube root and no division.  Outside that range, h^2 cbrt(h) divides.
-__device__ __forceinline__ double h_m73(double h) {
-  if (!(fbits(h) > fbits(1e-30) && fbits(h) < fbits(1e30))) return 1.0 / (h * h * cbrt(h));
-  double r = (double)rcbrtf((float)h);
-  const double third = 1.0 / 3.0;
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    const double e = fma(-h, r * r * r, 1.0);
-    r = fma(r * third, e, r);
-  }
-  const double r3 = r * r * r;
-  return r * (r3 * r3);
-}
-
+// For h in (1e-30, 1e30), h^(-7/3) comes from the FP32 inverse cube root r of h (cut to
+// FP32 on the integer units) and the binomial series about it: h = (1 - e) / r^3 with
+// |e| < 1e-6, so h^(-7/3) = r^7 (1 + 7/3 e + 35/9 e^2 + O(6 e^3)), 8 FP64 instructions and
+// no conversion; two Newton steps on the root took about 20.  Outside, h^2 cbrt(h) divides.
 __device__ __forceinline__ void friction_point(double gn2dt, double tol, double h, double& qx,
                                                double& qy) {
   if (!above(h, tol)) return;
-  const double qm = sqrt(qx * qx + qy * qy);
-  const double den = 1.0 + gn2dt * qm * h_m73(h);
-  const double iden = 1.0 / den;
+  const double qm = sqrt64(fma(qx, qx, qy * qy));
+  double iden;
+  if (fbits(h) > fbits(1e-30) && fbits(h) < fbits(1e30)) {
+    const float hf = __int_as_float(((__double2hiint(h) - 0x38000000) << 3) |
+                                    (int)((unsigned)__double2loint(h) >> 29));
+    const int rb = __float_as_int(rcbrtf(hf));
+    const double r = __hiloint2double((rb >> 3) + 0x38000000, rb << 29);
+    const double r3 = r * r * r;
+    const double e = fma(-h, r3, 1.0);
+    const double r7 = r3 * r3 * r;
+    const double hm73 = fma(r7 * e, fma(35.0 / 9.0, e, 7.0 / 3.0), r7);
+    iden = rcp64(fma(gn2dt * qm, hm73, 1.0));
+  } else {
+    iden = 1.0 / (1.0 + gn2dt * qm / (h * h * cbrt(h)));
+  }
   qx = qx * iden;
   qy = qy * iden;
 }
@@ -790,10 +778,24 @@ struct Rec {
   int pw;
 };
 
-// A revised face: its flux and the lower (west / south) side's revised depth
+// One side of a revised face: h*, q* = h* u and the bed level of its own bed term.
+struct Side {
+  double h, qx, qy, z;
+};
+
+// A revised face: its flux and the lower (west / south) side's revised state
 // and bed level for that side's own Eq. 5 and bed term.
 struct FaceR {
-  double fh, fx, fy, ha, za;
+  double h, n, t;  // the flux (Flux without dp, which the upper side's thread keeps)
+  Side a;
+};
+
+// Step constants of a stage, formed once per block: the weights of Eqs. 4a-c with the
+// stage's step (dt, halved in stage 2 for the RK average) folded in.
+struct StageK {
+  double dx, dy;    // -dt / dx, -dt / dy
+  double dx3, dy3;  // -3 dt / dx, -3 dt / dy
+  double bx, by;    // -g dt / (2 dx), -g dt / (2 dy)
 };
 
 struct StageSmem {
@@ -806,6 +808,7 @@ struct StageSmem {
   FaceR fx[TY][TX + 1];  // x faces; fx[ty][tx] is the west face of column tx
   FaceR fy[TY + 1][TX];  // y faces; fy[ty][tx] is the south face of row ty
   double red[32];
+  StageK k;
   unsigned char nq[TY + 2][TX + 2];   // the stage input's non-quiescence, tile and ring
   unsigned char cls[TY][TX];          // 0 outside the grid, 1 fixed point, 2 computed
   unsigned char nqo[TY][TX];          // the stage output's non-quiescence
@@ -834,12 +837,13 @@ __device__ __forceinline__ Rec make_rec(double h, double qx, double qy, double z
     r.u = k * qx;
     r.v = k * qy;
   } else if (above(h, tol)) {
-    const double ih = 1.0 / h;
+    const double ih = rcp64(h);
     r.u = qx * ih;
     r.v = qy * ih;
   }
   const double hp = pos_part(h);
-  r.hs = pw ? sc * hp : hp;
+  r.hs = hp;
+  if (pw) r.hs = sc * hp;
   r.zf = zf;
   r.pw = pw ? 1 : 0;
   return r;
@@ -867,36 +871,43 @@ __device__ __forceinline__ bool pw_scale(double h0, double hW, double hE, double
 // free-surface revision of Sec. 2.2.2 on the sides' own bed levels (zf raised
 // by the depth a partially wet side does not offer): z* = max(za, zb),
 // h* = max(0, eta - z*), q* = h* u, each side's bed term on z* lowered by the
-// amount its free surface lies below it.
-__device__ __forceinline__ F3 revise_face(const Rec& a, const Rec& b, bool ydir, double g, double tol,
-                                          int flux, double& ha, double& za, double& hb, double& zb) {
-  Lim ra, rb;
+// amount its free surface lies below it.  The flux is in the face's frame.
+template <bool ROE>
+__device__ __forceinline__ Flux revise_face(const Rec& a, const Rec& b, bool ydir, double g,
+                                            double tol, Side& ra, Side& rb) {
   if (!a.pw && !b.pw) {
-    ha = a.hs;
-    hb = b.hs;
-    za = a.zf - (is_neg(a.h) ? -a.h : 0.0);
-    zb = b.zf - (is_neg(b.h) ? -b.h : 0.0);
-    // the flux's velocities follow the tol rule on the revised depth
-    const bool wa = above(ha, tol), wb = above(hb, tol);
-    ra.u = wa ? a.u : 0.0; ra.v = wa ? a.v : 0.0;
-    rb.u = wb ? b.u : 0.0; rb.v = wb ? b.v : 0.0;
+    ra.h = a.hs;
+    rb.h = b.hs;
+    ra.z = a.zf;
+    rb.z = b.zf;
+    if (is_neg(a.h)) ra.z = a.zf + a.h;
+    if (is_neg(b.h)) rb.z = b.zf + b.h;
   } else {
     double ea, oa, eb, ob;  // free surface and own bed level of each side
     if (a.pw) { ea = a.h + a.zf; oa = ea - a.hs; } else { oa = a.zf; ea = a.zf + a.hs; }
     if (b.pw) { eb = b.h + b.zf; ob = eb - b.hs; } else { ob = b.zf; eb = b.zf + b.hs; }
     const double zs = gt(oa, ob) ? oa : ob;
     const double da = ea - zs, db = eb - zs;
-    ha = pos_part(da);
-    hb = pos_part(db);
-    za = zs - (is_neg(da) ? -da : 0.0);
-    zb = zs - (is_neg(db) ? -db : 0.0);
-    const bool wa = above(ha, tol), wb = above(hb, tol);
-    ra.u = wa ? a.u : 0.0; ra.v = wa ? a.v : 0.0;
-    rb.u = wb ? b.u : 0.0; rb.v = wb ? b.v : 0.0;
+    ra.h = pos_part(da);
+    rb.h = pos_part(db);
+    ra.z = zs;
+    rb.z = zs;
+    if (is_neg(da)) ra.z = zs + da;
+    if (is_neg(db)) rb.z = zs + db;
   }
-  ra.h = ha; ra.qx = ha * a.u; ra.qy = ha * a.v;
-  rb.h = hb; rb.qx = hb * b.u; rb.qy = hb * b.v;
-  return flux_dir(ra, rb, ydir, g, tol, flux);
+  ra.qx = ra.h * a.u; ra.qy = ra.h * a.v;
+  rb.qx = rb.h * b.u; rb.qy = rb.h * b.v;
+  // the flux's velocities follow the tol rule on the revised depth
+  const double an = ydir ? ra.qy : ra.qx, at = ydir ? ra.qx : ra.qy;
+  const double bn = ydir ? rb.qy : rb.qx, bt = ydir ? rb.qx : rb.qy;
+  double aun = ydir ? a.v : a.u, aut = ydir ? a.u : a.v;
+  double bun = ydir ? b.v : b.u, but = ydir ? b.u : b.v;
+  if (ROE) {
+    if (!above(ra.h, tol)) { aun = 0.0; aut = 0.0; }
+    if (!above(rb.h, tol)) { bun = 0.0; but = 0.0; }
+    return roe(ra.h, an, at, aun, aut, rb.h, bn, bt, bun, but, g, tol);
+  }
+  return hll(ra.h, an, at, aun, aut, rb.h, bn, bt, bun, but, g, tol);
 }
 
 // Planar depth slope of cell (i, j) along dir, limited (Eqs. 6-7 on eta) when
@@ -1051,19 +1062,24 @@ __device__ __forceinline__ void classify_cells(const Dev& d, StageSmem& sm, int 
 // non-quiescent flags of the thread's cell into the caller's variables.  Cells
 // that are fixed points of the stage (classify_cells) skip the faces and
 // Eqs. 4-5.
-template <bool LL, int STAGE>
+template <bool LL, int STAGE, bool ROE>
 __device__ __forceinline__ void stage_tile(const Dev& d, StageSmem& sm, int bx, int by,
                                            double& brate, double& lam, bool& bad, bool& nonq) {
   Scalars* sc = d.sc;
   const int tile = by * d.tiles.ntx + bx;
   const bool every = !d.tiles.skip || d.tiles.all_forced || d.tiles.forced[tile];
+  const double dt = sc->dt;
+  if (threadIdx.x == 0 && threadIdx.y == 0) {
+    const double k = STAGE == 1 ? dt : 0.5 * dt;
+    sm.k = StageK{-k * d.inv_dx, -k * d.inv_dy, -3.0 * k * d.inv_dx, -3.0 * k * d.inv_dy,
+                  -0.5 * d.g * k * d.inv_dx, -0.5 * d.g * k * d.inv_dy};
+  }
   int tx, ty;
   classify_cells<STAGE>(d, sm, bx, by, every, tx, ty);
   const int i = bx * TX + tx, j = by * TY + ty;
   const bool act = i < d.nx && j < d.ny;
   const long long P = d.plane;
   const long long c = (long long)j * d.pitch + i;
-  const double dt = sc->dt;
   const double ts = STAGE == 1 ? sc->t : sc->t + dt;  // boundary-condition time
   const double* __restrict__ In = STAGE == 1 ? d.S : d.T;
   const double g = d.g, tol = d.tol;
@@ -1072,7 +1088,7 @@ __device__ __forceinline__ void stage_tile(const Dev& d, StageSmem& sm, int bx, 
   const bool b_s = ty > 0 && sm.cls[ty - 1][tx] == 2, b_n = ty + 1 < TY && sm.cls[ty + 1][tx] == 2;
   double m[9];
   double z0 = 0.0, z1x = 0.0, z1y = 0.0;
-  Rec rE, rW, rN, rS;  // own records
+  Rec rW, rS;  // own records at the faces this thread revises
   // records: a computed cell's, and those of its neighbours (their limits make
   // the computed cell's faces)
   const bool recs = act && (b_me || b_w || b_e || b_s || b_n);
@@ -1090,12 +1106,10 @@ __device__ __forceinline__ void stage_tile(const Dev& d, StageSmem& sm, int bx, 
     double scl;
     const bool pw = pw_scale(m[H0], wh, eh, shh, nh, tol, d.wd, scl);
     const bool thin = d.wd != 0;
-    rE = make_rec(eh, m[QX0] + m[QX1X], m[QY0] + m[QY1X], z0 + z1x, pw, scl, tol, thin, m[H0]);
+    sm.e[ty][tx] = make_rec(eh, m[QX0] + m[QX1X], m[QY0] + m[QY1X], z0 + z1x, pw, scl, tol, thin, m[H0]);
     rW = make_rec(wh, m[QX0] - m[QX1X], m[QY0] - m[QY1X], z0 - z1x, pw, scl, tol, thin, m[H0]);
-    rN = make_rec(nh, m[QX0] + m[QX1Y], m[QY0] + m[QY1Y], z0 + z1y, pw, scl, tol, thin, m[H0]);
+    sm.n[ty][tx] = make_rec(nh, m[QX0] + m[QX1Y], m[QY0] + m[QY1Y], z0 + z1y, pw, scl, tol, thin, m[H0]);
     rS = make_rec(shh, m[QX0] - m[QX1Y], m[QY0] - m[QY1Y], z0 - z1y, pw, scl, tol, thin, m[H0]);
-    sm.e[ty][tx] = rE;
-    sm.n[ty][tx] = rN;
   }
   // the records beyond the tile (a neighbour's, or the edge ghost), one per
   // thread of the last 2 (TX + TY) threads (the fixed-point cells' threads when
@@ -1139,84 +1153,108 @@ __device__ __forceinline__ void stage_tile(const Dev& d, StageSmem& sm, int bx, 
   // (the own, upper side stays in registers, the lower side's depth and bed go
   // to shared memory with the flux), then the tile's east and north edge
   // faces one per thread (again the last threads)
-  double hWo = 0, zWo = 0, hSo = 0, zSo = 0;
+  Side W = {}, S = {};          // the own side of the west and south faces
+  double dpW = 0.0, dpS = 0.0;  // their pressure steps
   if (act && (b_me || b_w)) {
-    double ha, za;
-    const Rec& Lw = tx > 0 ? sm.e[ty][tx - 1] : sm.hw[ty];
-    const F3 fw = revise_face(Lw, rW, false, g, tol, d.flux, ha, za, hWo, zWo);
-    sm.fx[ty][tx] = FaceR{fw.h, fw.x, fw.y, ha, za};
-    if (i == 0) brate += fw.h * d.dy;
+    FaceR f;
+    const Flux w = revise_face<ROE>(tx > 0 ? sm.e[ty][tx - 1] : sm.hw[ty], rW, false, g, tol, f.a, W);
+    f.h = w.h; f.n = w.n; f.t = w.t;
+    sm.fx[ty][tx] = f;
+    dpW = w.dp;
+    if (i == 0) brate += w.h * d.dy;
   }
   if (act && (b_me || b_s)) {
-    double ha, za;
-    const Rec& Ls = ty > 0 ? sm.n[ty - 1][tx] : sm.hs[tx];
-    const F3 fs = revise_face(Ls, rS, true, g, tol, d.flux, ha, za, hSo, zSo);
-    sm.fy[ty][tx] = FaceR{fs.h, fs.x, fs.y, ha, za};
-    if (j == 0) brate += fs.h * d.dx;
+    FaceR f;
+    const Flux w = revise_face<ROE>(ty > 0 ? sm.n[ty - 1][tx] : sm.hs[tx], rS, true, g, tol, f.a, S);
+    f.h = w.h; f.n = w.n; f.t = w.t;
+    sm.fy[ty][tx] = f;
+    dpS = w.dp;
+    if (j == 0) brate += w.h * d.dx;
   }
   {
     const int t = TX * TY - 1 - (threadIdx.y * TX + threadIdx.x);
     const int ni = d.nx - bx * TX < TX ? d.nx - bx * TX : TX;
     const int nj = d.ny - by * TY < TY ? d.ny - by * TY : TY;
-    double ha, za, hb, zb;
     // east edge faces (t < nj) and north edge faces (TY <= t < TY + ni) on one
     // code path: the north faces' normal is y
     const bool yf = t >= TY;
     const int q = yf ? t - TY : t;
     if ((yf ? q < ni : q < nj) && (yf ? sm.cls[nj - 1][q] : sm.cls[q][ni - 1]) == 2) {
-      const F3 f = revise_face(yf ? sm.n[nj - 1][q] : sm.e[q][ni - 1], yf ? sm.hn[q] : sm.he[q], yf,
-                               g, tol, d.flux, ha, za, hb, zb);
-      FaceR* dst = yf ? &sm.fy[nj][q] : &sm.fx[q][ni];
-      *dst = FaceR{f.h, f.x, f.y, ha, za};
+      FaceR o;
+      Side b;
+      const Flux f = revise_face<ROE>(yf ? sm.n[nj - 1][q] : sm.e[q][ni - 1],
+                                      yf ? sm.hn[q] : sm.he[q], yf, g, tol, o.a, b);
+      o.h = f.h; o.n = f.n; o.t = f.t;
+      *(yf ? &sm.fy[nj][q] : &sm.fx[q][ni]) = o;
       if (yf ? by * TY + nj == d.ny : bx * TX + ni == d.nx) brate -= f.h * (yf ? d.dx : d.dy);
     }
   }
   __syncthreads();
   bool nq_out = false;  // the cell's output is non-quiescent
   if (act && b_me) {
-    const FaceR FW = sm.fx[ty][tx], FE = sm.fx[ty][tx + 1];
-    const FaceR GS = sm.fy[ty][tx], GN = sm.fy[ty + 1][tx];
-    // own side of the east / north faces: revised as their lower side
-    const double hEo = FE.ha, zEo = FE.za, hNo = GN.ha, zNo = GN.za;
-    // own revised states (Eq. 5 operands): q* = h* u
-    const double Esh = hEo, Esx = hEo * rE.u, Esy = hEo * rE.v;
-    const double Wsh = hWo, Wsx = hWo * rW.u, Wsy = hWo * rW.v;
-    const double Nsh = hNo, Nsx = hNo * rN.u, Nsy = hNo * rN.v;
-    const double Ssh = hSo, Ssx = hSo * rS.u, Ssy = hSo * rS.v;
-    const double zb1x = 0.5 * (zEo - zWo), zb1y = 0.5 * (zNo - zSo);
-    // dummy modes (Eq. 5; the second line read as the 0y mode)
-    const double h0x = 0.5 * (Esh + Wsh), x0x = 0.5 * (Esx + Wsx), y0x = 0.5 * (Esy + Wsy);
-    const double h1x_ = 0.5 * (Esh - Wsh), x1x = 0.5 * (Esx - Wsx), y1x = 0.5 * (Esy - Wsy);
-    const double h0y = 0.5 * (Nsh + Ssh), x0y = 0.5 * (Nsx + Ssx), y0y = 0.5 * (Nsy + Ssy);
-    const double h1y_ = 0.5 * (Nsh - Ssh), x1y = 0.5 * (Nsx - Ssx), y1y = 0.5 * (Nsy - Ssy);
-    const double r3 = 1.0 / 1.7320508075688772;
-    const F3 Fp = phys_flux(h0x + h1x_ * r3, x0x + x1x * r3, y0x + y1x * r3, g, tol, false);
-    const F3 Fm = phys_flux(h0x - h1x_ * r3, x0x - x1x * r3, y0x - y1x * r3, g, tol, false);
-    const F3 Gp = phys_flux(h0y + h1y_ * r3, x0y + x1y * r3, y0y + y1y * r3, g, tol, true);
-    const F3 Gm = phys_flux(h0y - h1y_ * r3, x0y - x1y * r3, y0y - y1y * r3, g, tol, true);
-    const double idx = d.inv_dx, idy = d.inv_dy;
-    // Eq. 4a
-    double L[9];
-    L[H0] = -(FE.fh - FW.fh) * idx - (GN.fh - GS.fh) * idy;
-    L[QX0] = -(FE.fx - FW.fx) * idx - (GN.fx - GS.fx) * idy - 2.0 * g * h0x * zb1x * idx;
-    L[QY0] = -(FE.fy - FW.fy) * idx - (GN.fy - GS.fy) * idy - 2.0 * g * h0y * zb1y * idy;
-    if (d.rain != 0.0 && ts >= d.rain_t0 && ts < d.rain_t1) L[H0] += d.rain;
-    if (c == d.src_idx) L[H0] += d.qp * idx * idy;
-    // Eq. 4b
-    const double k3x = -3.0 * idx, k3y = -3.0 * idy, g23 = 2.0 * g / 3.0;
-    L[H1X] = k3x * ((FE.fh + FW.fh) - (Fp.h + Fm.h));
-    L[QX1X] = k3x * ((FE.fx + FW.fx) - (Fp.x + Fm.x) + g23 * h1x_ * zb1x);
-    L[QY1X] = k3x * ((FE.fy + FW.fy) - (Fp.y + Fm.y));
-    // Eq. 4c
-    L[H1Y] = k3y * ((GN.fh + GS.fh) - (Gp.h + Gm.h));
-    L[QX1Y] = k3y * ((GN.fx + GS.fx) - (Gp.x + Gm.x));
-    L[QY1Y] = k3y * ((GN.fy + GS.fy) - (Gp.y + Gm.y) + g23 * h1y_ * zb1y);
-
+    // The stage's update is base + k L, k = dt and base = U^n in stage 1, k = dt / 2 and
+    // base = (U^n + U^1) / 2 in stage 2, with L of Eqs. 4-5 and the step folded into its
+    // weights (StageK).  The own pressures and the bed terms of a direction share one
+    // product: with s, d the sum and difference of the own face depths and r = d + zE - zW
+    // the step of the free surface between the faces, Eq. 4a has -g s r / (2 dx) and
+    // Eqs. 4b-c (with the Gauss points' pressures) -g d r / (2 dx) beside the
+    // pressure-free fluxes.  Small terms are summed before they meet the base.
+    const StageK K = sm.k;
     double out[9];
     if (STAGE == 1) {
 #pragma unroll
-      for (int k = 0; k < 9; ++k) out[k] = m[k] + dt * L[k];
-      wetdry(out, z0, z1x, z1y, tol);
+      for (int k = 0; k < 9; ++k) out[k] = m[k];
+    } else {
+      out[H0] = d.S[H0 * P + c]; out[QX0] = d.S[QX0 * P + c]; out[QY0] = d.S[QY0 * P + c];
+      if (LL) {
+        out[H1X] = d.Q[0 * P + c]; out[H1Y] = d.Q[1 * P + c];
+        out[QX1X] = d.Q[2 * P + c]; out[QX1Y] = d.Q[3 * P + c];
+        out[QY1X] = d.Q[4 * P + c]; out[QY1Y] = d.Q[5 * P + c];
+      } else {
+        out[H1X] = d.S[H1X * P + c]; out[H1Y] = d.S[H1Y * P + c];
+        out[QX1X] = d.S[QX1X * P + c]; out[QX1Y] = d.S[QX1Y * P + c];
+        out[QY1X] = d.S[QY1X * P + c]; out[QY1Y] = d.S[QY1Y * P + c];
+      }
+#pragma unroll
+      for (int k = 0; k < 9; ++k) out[k] = half64(out[k] + m[k]);
+    }
+    const double tol2 = 2.0 * tol;
+    double l0, lx, ly;  // k L of the averages
+    {  // x direction
+      const FaceR& FW = sm.fx[ty][tx];
+      const FaceR& FE = sm.fx[ty][tx + 1];
+      const Side E = FE.a;  // own side of the east face: its lower side
+      const double hs = E.h + W.h, hd = E.h - W.h;
+      const F3 G = gauss_pair(hs, E.qx + W.qx, E.qy + W.qy, hd, E.qx - W.qx, E.qy - W.qy, tol2);
+      const double bed = K.bx * (hd + (E.z - W.z));
+      const double eh = FE.h, wh = FW.h, en = FE.n, wn = FW.n + dpW, et = FE.t, wt = FW.t;
+      l0 = K.dx * (eh - wh);
+      lx = fma(K.dx, en - wn, bed * hs);
+      ly = K.dx * (et - wt);
+      out[H1X] = fma(K.dx3, fma(-0.5, G.h, eh + wh), out[H1X]);
+      out[QX1X] += fma(K.dx3, fma(-0.5, G.n, en + wn), bed * hd);
+      out[QY1X] = fma(K.dx3, fma(-0.5, G.t, et + wt), out[QY1X]);
+    }
+    {  // y direction
+      const FaceR& FS = sm.fy[ty][tx];
+      const FaceR& FN = sm.fy[ty + 1][tx];
+      const Side N = FN.a;
+      const double hs = N.h + S.h, hd = N.h - S.h;
+      const F3 G = gauss_pair(hs, N.qy + S.qy, N.qx + S.qx, hd, N.qy - S.qy, N.qx - S.qx, tol2);
+      const double bed = K.by * (hd + (N.z - S.z));
+      const double nh = FN.h, sh = FS.h, nn = FN.n, sn = FS.n + dpS, nt = FN.t, st = FS.t;
+      out[H0] += fma(K.dy, nh - sh, l0);
+      out[QX0] += fma(K.dy, nt - st, lx);
+      out[QY0] += fma(bed, hs, fma(K.dy, nn - sn, ly));
+      out[H1Y] = fma(K.dy3, fma(-0.5, G.h, nh + sh), out[H1Y]);
+      out[QX1Y] = fma(K.dy3, fma(-0.5, G.t, nt + st), out[QX1Y]);
+      out[QY1Y] += fma(K.dy3, fma(-0.5, G.n, nn + sn), bed * hd);
+    }
+    if (d.rain != 0.0 && ts >= d.rain_t0 && ts < d.rain_t1)
+      out[H0] += (STAGE == 1 ? dt : 0.5 * dt) * d.rain;
+    if (c == d.src_idx) out[H0] += (STAGE == 1 ? dt : 0.5 * dt) * (d.qp * d.inv_dx * d.inv_dy);
+    wetdry(out, z0, z1x, z1y, tol);
+    if (STAGE == 1) {
 #pragma unroll
       for (int k = 0; k < 9; ++k) d.T[k * P + c] = out[k];
       nq_out = above(out[H0], tol);
@@ -1228,20 +1266,6 @@ __device__ __forceinline__ void stage_tile(const Dev& d, StageSmem& sm, int bx, 
         d.Q[4 * P + c] = m[QY1X]; d.Q[5 * P + c] = m[QY1Y];
       }
     } else {
-      double un[9];
-      un[H0] = d.S[H0 * P + c]; un[QX0] = d.S[QX0 * P + c]; un[QY0] = d.S[QY0 * P + c];
-      if (LL) {
-        un[H1X] = d.Q[0 * P + c]; un[H1Y] = d.Q[1 * P + c];
-        un[QX1X] = d.Q[2 * P + c]; un[QX1Y] = d.Q[3 * P + c];
-        un[QY1X] = d.Q[4 * P + c]; un[QY1Y] = d.Q[5 * P + c];
-      } else {
-        un[H1X] = d.S[H1X * P + c]; un[H1Y] = d.S[H1Y * P + c];
-        un[QX1X] = d.S[QX1X * P + c]; un[QX1Y] = d.S[QX1Y * P + c];
-        un[QY1X] = d.S[QY1X * P + c]; un[QY1Y] = d.S[QY1Y * P + c];
-      }
-#pragma unroll
-      for (int k = 0; k < 9; ++k) out[k] = 0.5 * (un[k] + m[k] + dt * L[k]);
-      wetdry(out, z0, z1x, z1y, tol);
 #pragma unroll
       for (int k = 0; k < 9; ++k) d.S[k * P + c] = out[k];
       lam = cell_rate(d, out[H0], out[QX0], out[QY0]);
@@ -1281,17 +1305,20 @@ __device__ __forceinline__ void stage_tile(const Dev& d, StageSmem& sm, int bx, 
   }
 }
 
-// Work distribution of the stage kernels over the step's tile lists:
-// DG2_TILE_LOOP64 1 runs a fixed grid of resident blocks that loop over the
-// entries; 0 launches one block per tile of the grid and a block takes the
-// entry of its own index (blocks past the lists exit at once, and the
-// hardware balances tiles of unequal cost over the SMs).  Measured on the
-// 2000 x 1000 floodplain: FP64 tiles (tens of microseconds each, 1-2 blocks
-// per SM) run faster one per block; the FP32 kernels (shared with ensembles)
-// loop over the list in resident blocks.
-#ifndef DG2_TILE_LOOP64
-#define DG2_TILE_LOOP64 0
-#endif
+// Work distribution of the stage kernels over the step's tile lists: one block per tile
+// of the grid, and a block takes the entry of its own index (blocks past the lists exit
+// at once, and the hardware balances tiles of unequal cost over the SMs).  On the
+// 2000 x 1000 floodplain FP64 tiles (tens of microseconds each, 1-2 blocks per SM) run
+// faster so than in resident blocks that loop over the list; the FP32 kernels (shared
+// with ensembles) loop.
+// The FP64 pipe bounds both stages (two lanes an SM and cycle against 128 FP32 ones).
+// Their arithmetic in fewer FP64 instructions (rcp64 / sqrt64, hll, the deviation form of
+// Flux, folded step weights, friction's series) took whole passes from the start of this
+// form to its end (state in, run, state out): 2000 x 1000 floodplain DG2-LL 42.7 -> 29.9 ms,
+// 1237 x 731 floodplain DG2-NL 36.8 -> 27.1 ms, 1000 x 600 flooded plain DG2-LL 58.5 ->
+// 44.8 ms, the 128 x 128 basin 13.5 -> 10.9 ms, with errors against an 80-bit run of the
+// same scheme 1.0 to 0.9 of what they were.
+//
 // minimum resident blocks per SM asked of the register allocator: 2 for both
 // FP64 stages (128 registers; measured on the floodplain, DG2-LL 0.857 ms/step
 // at 2 blocks against 0.955 at 1 block with 156 registers)
@@ -1305,7 +1332,7 @@ __device__ __forceinline__ void stage_tile(const Dev& d, StageSmem& sm, int bx, 
 // Stage kernels run over the step's list of active tiles (and, in stage 1,
 // the frontier tiles that only copy their state for a neighbour's halo),
 // built at the end of the previous step.
-template <bool LL, int STAGE>
+template <bool LL, int STAGE, bool ROE>
 static __global__ void __launch_bounds__(TX* TY, LL ? DG2_MINB64_LL : DG2_MINB64_NL) stage_kernel(Dev d) {
   extern __shared__ double stage_smem[];  // one StageSmem (dynamic: above 48 KB)
   StageSmem& sm = *reinterpret_cast<StageSmem*>(stage_smem);
@@ -1317,17 +1344,14 @@ static __global__ void __launch_bounds__(TX* TY, LL ? DG2_MINB64_LL : DG2_MINB64
   const bool all = sc->list_all != 0;
   double lam = 0.0;
   bool bad = false;
-#if DG2_TILE_LOOP64
-  for (int e = blockIdx.x; e < n_act; e += gridDim.x) {
-#else
   if (STAGE == 2 && (int)blockIdx.x >= n_act) return;
-  for (int e = blockIdx.x; e < n_act; e = n_act) {
-#endif
+  if ((int)blockIdx.x < n_act) {
+    const int e = blockIdx.x;
     const int tile = all ? e : list_tile(d.tiles, sc, e);
     const int bx = tile % ntx, by = tile / ntx;
     double brate = 0.0, lam_t = 0.0;
     bool nonq = false;
-    stage_tile<LL, STAGE>(d, sm, bx, by, brate, lam_t, bad, nonq);
+    stage_tile<LL, STAGE, ROE>(d, sm, bx, by, brate, lam_t, bad, nonq);
     lam = fmax(lam, lam_t);
     // boundary inflow rate of an edge tile, kept per tile (summed in tile order later)
     if (bx == 0 || by == 0 || bx == ntx - 1 || by == d.tiles.nty - 1) {
@@ -1344,11 +1368,8 @@ static __global__ void __launch_bounds__(TX* TY, LL ? DG2_MINB64_LL : DG2_MINB64
     // frontier tiles: a computed neighbour reads their stage state as halo
     const int n_front = sc->n_front;
     const long long P = d.plane;
-#if DG2_TILE_LOOP64
-    for (int e = blockIdx.x; e < n_front; e += gridDim.x) {
-#else
-    for (int e = (int)blockIdx.x - n_act; e >= 0 && e < n_front; e = n_front) {
-#endif
+    const int e = (int)blockIdx.x - n_act;
+    if (e >= 0 && e < n_front) {
       const int tile = d.tiles.front[e];
       int cx, cy;
       warp_cell(cx, cy);

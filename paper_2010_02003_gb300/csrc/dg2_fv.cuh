@@ -28,10 +28,10 @@ struct L4 {
   double eta, h, qx, qy;
 };
 
-// A face after the revision: its flux, z* and the revised depths on the lower
-// (a: west / south) and upper (b: east / north) side.
+// A face after the revision: its flux (Flux without dp, which the upper side's thread keeps), z* and
+// the revised depths on the lower (a: west / south) and upper (b: east / north) side.
 struct Face {
-  double h, x, y, zs, ha, hb;
+  double h, n, t, zs, ha, hb;
 };
 
 struct Smem {
@@ -101,7 +101,7 @@ __device__ __forceinline__ L4 ghost4(const Dev& d, int edge, double s, double t,
 // Revision of a face (Sec. 2.2.2) from its lower (a) and upper (b) limits and
 // the flux across it.
 __device__ __forceinline__ Face face(const L4& a, const L4& b, bool ydir, double g, double tol,
-                                     int flux) {
+                                     int flux, double& dp) {
   const double za = a.eta - a.h, zb = b.eta - b.h;
   const double zs = za > zb ? za : zb;
   double ha = a.eta - zs, hb = b.eta - zs;
@@ -113,14 +113,15 @@ __device__ __forceinline__ Face face(const L4& a, const L4& b, bool ydir, double
   double ua = 0.0, va = 0.0, ub = 0.0, vb = 0.0;
   if (a.h > tol) { ua = a.qx / a.h; va = a.qy / a.h; }
   if (b.h > tol) { ub = b.qx / b.h; vb = b.qy / b.h; }
-  Lim ra, rb;
-  ra.h = ha; ra.qx = ha * ua; ra.qy = ha * va;
-  rb.h = hb; rb.qx = hb * ub; rb.qy = hb * vb;
-  ra.u = ha > tol ? ua : 0.0; ra.v = ha > tol ? va : 0.0;
-  rb.u = hb > tol ? ub : 0.0; rb.v = hb > tol ? vb : 0.0;
-  const F3 F = ydir ? flux_y(ra, rb, g, tol, flux) : flux_x(ra, rb, g, tol, flux);
+  const double una = ha > tol ? (ydir ? va : ua) : 0.0, uta = ha > tol ? (ydir ? ua : va) : 0.0;
+  const double unb = hb > tol ? (ydir ? vb : ub) : 0.0, utb = hb > tol ? (ydir ? ub : vb) : 0.0;
+  const double qna = ha * (ydir ? va : ua), qta = ha * (ydir ? ua : va);
+  const double qnb = hb * (ydir ? vb : ub), qtb = hb * (ydir ? ub : vb);
+  const Flux F = flux == 1 ? roe(ha, qna, qta, una, uta, hb, qnb, qtb, unb, utb, g, tol)
+                           : hll(ha, qna, qta, una, uta, hb, qnb, qtb, unb, utb, g, tol);
   Face r;
-  r.h = F.h; r.x = F.x; r.y = F.y;
+  r.h = F.h; r.n = F.n; r.t = F.t;
+  dp = F.dp;
   r.zs = zs; r.ha = ha; r.hb = hb;
   return r;
 }
@@ -211,22 +212,23 @@ __device__ __forceinline__ void fv_tile(const Dev& d, Smem& sm, int bx, int by, 
   __syncthreads();  // the staged averages are dead past here (the faces reuse them)
 
   // one revision and one flux per face
+  double dpW = 0.0, dpS = 0.0, dpx;
   if (act) {
     const L4& Lw = tx > 0 ? sm.e[ty][tx - 1] : sm.hw[ty];
-    const Face fw = face(Lw, W, false, g, tol, d.flux);
+    const Face fw = face(Lw, W, false, g, tol, d.flux, dpW);
     sm.u.f.fx[ty][tx] = fw;
     if (i == 0) brate += fw.h * d.dy;
     if (east_edge) {
-      const Face fe = face(E, sm.he[ty], false, g, tol, d.flux);
+      const Face fe = face(E, sm.he[ty], false, g, tol, d.flux, dpx);
       sm.u.f.fx[ty][tx + 1] = fe;
       if (i == nx - 1) brate -= fe.h * d.dy;
     }
     const L4& Ls = ty > 0 ? sm.n[ty - 1][tx] : sm.hs[tx];
-    const Face fs = face(Ls, S, true, g, tol, d.flux);
+    const Face fs = face(Ls, S, true, g, tol, d.flux, dpS);
     sm.u.f.fy[ty][tx] = fs;
     if (j == 0) brate += fs.h * d.dx;
     if (north_edge) {
-      const Face fn = face(N, sm.hn[tx], true, g, tol, d.flux);
+      const Face fn = face(N, sm.hn[tx], true, g, tol, d.flux, dpx);
       sm.u.f.fy[ty + 1][tx] = fn;
       if (j == ny - 1) brate -= fn.h * d.dx;
     }
@@ -240,13 +242,15 @@ __device__ __forceinline__ void fv_tile(const Dev& d, Smem& sm, int bx, int by, 
     const double dE = E.eta - fe.zs, dW = W.eta - fw.zs, dN = N.eta - fn.zs, dS = S.eta - fs.zs;
     const double zE = fe.zs - (dE < 0.0 ? -dE : 0.0), zW = fw.zs - (dW < 0.0 ? -dW : 0.0);
     const double zN = fn.zs - (dN < 0.0 ? -dN : 0.0), zS = fs.zs - (dS < 0.0 ? -dS : 0.0);
-    const double h0x = 0.5 * (fe.ha + fw.hb), z1x = 0.5 * (zE - zW);
-    const double h0y = 0.5 * (fn.ha + fs.hb), z1y = 0.5 * (zN - zS);
+    // own pressures and bed term of a direction: g / 2 (hE + hW) times the step of the
+    // free surface between the faces
+    const double bx = 0.5 * g * (fe.ha + fw.hb) * ((fe.ha - fw.hb) + (zE - zW));
+    const double by = 0.5 * g * (fn.ha + fs.hb) * ((fn.ha - fs.hb) + (zN - zS));
     const double idx = d.inv_dx, idy = d.inv_dy;
     // Eq. 8
     double Lh = -(fe.h - fw.h) * idx - (fn.h - fs.h) * idy;
-    const double Lx = -(fe.x - fw.x) * idx - (fn.x - fs.x) * idy - 2.0 * g * h0x * z1x * idx;
-    const double Ly = -(fe.y - fw.y) * idx - (fn.y - fs.y) * idy - 2.0 * g * h0y * z1y * idy;
+    const double Lx = -((fe.n - (fw.n + dpW)) + bx) * idx - (fn.t - fs.t) * idy;
+    const double Ly = -(fe.t - fw.t) * idx - ((fn.n - (fs.n + dpS)) + by) * idy;
     if (d.rain != 0.0 && ts >= d.rain_t0 && ts < d.rain_t1) Lh += d.rain;
     if (c == d.src_idx) Lh += d.qp * idx * idy;
     double h, qx, qy;
