@@ -704,6 +704,11 @@ __device__ __forceinline__ void friction_tile(const Dev& d, int bx, int by, unsi
   bool work = i < d.nx && j < d.ny;
   if (work && d.qm && d.tiles.skip && d.scheme == 0)
     work = (d.qm[(long long)(by * TBY + ty / WY) * d.nbx + bx * TBX + tx / WX] >> lane) & 1u;
+  if (work && d.scheme != 0) {
+    // the FV schemes keep no cell masks: a cell with no wet point by its depth modes
+    const long long c = (long long)j * d.pitch + i;
+    work = above(d.S[c], d.tol) || nonzero(d.S[P + c]) || nonzero(d.S[2 * P + c]);
+  }
   if (work) work = d.N[(long long)j * d.pitch + i] != 0.0;
   const unsigned bw = __ballot_sync(0xffffffffu, work);
   if (lane == 0) cnt[w] = __popc(bw);
@@ -732,6 +737,10 @@ __device__ __forceinline__ void friction_tile(const Dev& d, int bx, int by, unsi
 #pragma unroll
     for (int dd = 1; dd <= 2; ++dd) {
       const double h1 = S[dd * P + c], x1 = S[(3 + dd) * P + c], y1 = S[(6 + dd) * P + c];
+      nq[dd - 1][0] = 0.0;
+      nq[dd - 1][1] = 0.0;
+      // without slopes both Gauss points are the centre (the FV schemes, fronts)
+      if (!nonzero(h1) && !nonzero(x1) && !nonzero(y1)) continue;
       double xp = x0 + x1 * r3, yp = y0 + y1 * r3, xm = x0 - x1 * r3, ym = y0 - y1 * r3;
       friction_point(gn2dt, d.tol, h0 + h1 * r3, xp, yp);
       friction_point(gn2dt, d.tol, h0 - h1 * r3, xm, ym);

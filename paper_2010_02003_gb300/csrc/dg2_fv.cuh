@@ -12,10 +12,17 @@
 //
 // One block per 32 x 8 tile of the step's lists, as the DG2 stage kernels:
 // the averages of the tile and a 2-cell halo are staged in shared memory, each
-// thread forms its cell's four limits, the tile's edge threads form the limit
+// thread forms its cell's four limits, the tile's last threads form the limits
 // beyond the tile, and every face flux is evaluated once.  Dry-tile skipping
 // carries over unchanged: a still, dry cell among still, dry neighbours has zero
-// fluxes, and the dry reset removes the discharge its bed term makes.
+// fluxes, and the dry reset removes the discharge its bed term makes.  The same
+// holds for single cells, so a cell whose input and four neighbours are still and
+// dry (read off the staged averages) takes L = 0 and its faces are left out.
+//
+// The FP64 pipe bounds the kernels.  Divisions (Sweby's ratio, the velocities) and FP64
+// comparisons used to make up most of their FP64 instructions, and every cell of a
+// computed tile was evaluated: a pass of 70 FV2 steps of a 2000 x 1000 floodplain, 4 % wet,
+// took 43.1 ms with the state in and out, 20.4 ms without them.
 #pragma once
 #include "dg2_device.cuh"
 
@@ -28,10 +35,10 @@ struct L4 {
   double eta, h, qx, qy;
 };
 
-// A face after the revision: its flux (Flux without dp, which the upper side's thread keeps), z* and
-// the revised depths on the lower (a: west / south) and upper (b: east / north) side.
+// A face after the revision: its flux (in the face's frame, Flux) and the lower (west /
+// south) side's revised depth.
 struct Face {
-  double h, n, t, zs, ha, hb;
+  double h, n, t, dp, ha;
 };
 
 struct Smem {
@@ -46,13 +53,18 @@ struct Smem {
   L4 n[TY][TX];  // north limit of each cell
   L4 hw[TY], he[TY], hs[TX], hn[TX];  // limits beyond the tile (neighbour or ghost)
   double red[32];
+  StageK k;
+  unsigned char cls[TY][TX];  // 0 outside the grid, 1 L = 0, 2 computed
 };
 
-__device__ __forceinline__ double sweby(double r, double beta) {
-  const double a = beta * r < 1.0 ? beta * r : 1.0;
-  const double b = r < beta ? r : beta;
-  const double m = a > b ? a : b;
-  return m > 0.0 ? m : 0.0;
+// Slope of Eq. 10 with Sweby's limiter (beta = 1.25) from the backward and forward
+// differences: phi(fd / bd) bd without the division, max(min(beta |fd|, |bd|),
+// min(|fd|, beta |bd|)) with their sign where they share one, else 0.
+__device__ __forceinline__ double sweby_slope(double bd, double fd) {
+  if (!((is_pos(bd) && is_pos(fd)) || (is_neg(bd) && is_neg(fd)))) return 0.0;
+  const double a = fabs(fd), b = fabs(bd);
+  const double m = max_nn(min_nn(1.25 * a, b), min_nn(a, 1.25 * b));
+  return is_neg(bd) ? -m : m;
 }
 
 // Limited slopes (Eq. 10) of the four components of staged cell (a, b) along
@@ -64,12 +76,13 @@ __device__ __forceinline__ void slopes4(const double (*A)[HY][HX], int a, int b,
 #pragma unroll
   for (int k = 0; k < 4; ++k) s[k] = 0.0;
   if (!ORDER2 || edge) return;
-  if (A[1][b - db][a - da] <= tol || A[1][b][a] <= tol || A[1][b + db][a + da] <= tol) return;
+  if (!above(A[1][b - db][a - da], tol) || !above(A[1][b][a], tol) ||
+      !above(A[1][b + db][a + da], tol))
+    return;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const double vc = A[k][b][a];
-    const double bd = vc - A[k][b - db][a - da], fd = A[k][b + db][a + da] - vc;
-    s[k] = bd == 0.0 ? 0.0 : sweby(fd / bd, 1.25) * bd;
+    s[k] = sweby_slope(vc - A[k][b - db][a - da], A[k][b + db][a + da] - vc);
   }
 }
 
@@ -78,10 +91,10 @@ __device__ __forceinline__ void slopes4(const double (*A)[HY][HX], int a, int b,
 __device__ __forceinline__ L4 lim4(const double (*A)[HY][HX], int a, int b, const double s[4],
                                    double sg) {
   L4 r;
-  r.eta = A[0][b][a] + sg * s[0];
-  r.h = A[1][b][a] + sg * s[1];
-  r.qx = A[2][b][a] + sg * s[2];
-  r.qy = A[3][b][a] + sg * s[3];
+  r.eta = fma(sg, s[0], A[0][b][a]);
+  r.h = fma(sg, s[1], A[1][b][a]);
+  r.qx = fma(sg, s[2], A[2][b][a]);
+  r.qy = fma(sg, s[3], A[3][b][a]);
   return r;
 }
 
@@ -99,31 +112,38 @@ __device__ __forceinline__ L4 ghost4(const Dev& d, int edge, double s, double t,
 }
 
 // Revision of a face (Sec. 2.2.2) from its lower (a) and upper (b) limits and
-// the flux across it.
+// the flux across it; hb takes the upper side's revised depth.  h* + z* is the side's
+// own free surface on either side (z* lowered where the free surface lies below it), so
+// the update needs no bed levels (fv_tile).
 __device__ __forceinline__ Face face(const L4& a, const L4& b, bool ydir, double g, double tol,
-                                     int flux, double& dp) {
-  const double za = a.eta - a.h, zb = b.eta - b.h;
-  const double zs = za > zb ? za : zb;
-  double ha = a.eta - zs, hb = b.eta - zs;
-  if (ha < 0.0) ha = 0.0;
-  if (hb < 0.0) hb = 0.0;
+                                     int flux, double& hb) {
+  const double zs = max2(a.eta - a.h, b.eta - b.h);
+  const double ha = pos_part(a.eta - zs);
+  hb = pos_part(b.eta - zs);
   // q* = h* u with u of the limit (tol rule on the limit's depth); the flux
   // then takes its velocities from the revised state by the same rule, so a
   // face depth h* at or below tol_dry moves no water by advection
-  double ua = 0.0, va = 0.0, ub = 0.0, vb = 0.0;
-  if (a.h > tol) { ua = a.qx / a.h; va = a.qy / a.h; }
-  if (b.h > tol) { ub = b.qx / b.h; vb = b.qy / b.h; }
-  const double una = ha > tol ? (ydir ? va : ua) : 0.0, uta = ha > tol ? (ydir ? ua : va) : 0.0;
-  const double unb = hb > tol ? (ydir ? vb : ub) : 0.0, utb = hb > tol ? (ydir ? ub : vb) : 0.0;
-  const double qna = ha * (ydir ? va : ua), qta = ha * (ydir ? ua : va);
-  const double qnb = hb * (ydir ? vb : ub), qtb = hb * (ydir ? ub : vb);
-  const Flux F = flux == 1 ? roe(ha, qna, qta, una, uta, hb, qnb, qtb, unb, utb, g, tol)
-                           : hll(ha, qna, qta, una, uta, hb, qnb, qtb, unb, utb, g, tol);
-  Face r;
-  r.h = F.h; r.n = F.n; r.t = F.t;
-  dp = F.dp;
-  r.zs = zs; r.ha = ha; r.hb = hb;
-  return r;
+  double una = 0.0, uta = 0.0, unb = 0.0, utb = 0.0;
+  if (above(a.h, tol)) {
+    const double ih = rcp64(a.h);
+    una = (ydir ? a.qy : a.qx) * ih;
+    uta = (ydir ? a.qx : a.qy) * ih;
+  }
+  if (above(b.h, tol)) {
+    const double ih = rcp64(b.h);
+    unb = (ydir ? b.qy : b.qx) * ih;
+    utb = (ydir ? b.qx : b.qy) * ih;
+  }
+  const double qna = ha * una, qta = ha * uta, qnb = hb * unb, qtb = hb * utb;
+  Flux F;
+  if (flux == 1) {
+    if (!above(ha, tol)) { una = 0.0; uta = 0.0; }
+    if (!above(hb, tol)) { unb = 0.0; utb = 0.0; }
+    F = roe(ha, qna, qta, una, uta, hb, qnb, qtb, unb, utb, g, tol);
+  } else {
+    F = hll(ha, qna, qta, una, uta, hb, qnb, qtb, unb, utb, g, tol);
+  }
+  return Face{F.h, F.n, F.t, F.dp, ha};
 }
 
 // One FV stage on the 32 x 8 tile (bx, by).  Stage 1: T = S + dt L(S) (all
@@ -135,7 +155,9 @@ template <bool ORDER2, int STAGE>
 __device__ __forceinline__ void fv_tile(const Dev& d, Smem& sm, int bx, int by, double& brate,
                                         double& lam, bool& bad, bool& nonq) {
   const Scalars* sc = d.sc;
-  const int tx = threadIdx.x, ty = threadIdx.y;
+  const int tid = threadIdx.y * TX + threadIdx.x;
+  int tx, ty;
+  warp_cell(tx, ty);
   const int i0 = bx * TX, j0 = by * TY, i = i0 + tx, j = j0 + ty;
   const int nx = d.nx, ny = d.ny;
   const bool act = i < nx && j < ny;
@@ -144,9 +166,16 @@ __device__ __forceinline__ void fv_tile(const Dev& d, Smem& sm, int bx, int by, 
   const double ts = STAGE == 1 ? sc->t : sc->t + dt;
   const double* __restrict__ In = STAGE == 1 ? d.S : d.T;
   const double g = d.g, tol = d.tol;
+  const int tile = by * d.tiles.ntx + bx;
+  const bool every = !d.tiles.skip || d.tiles.all_forced || d.tiles.forced[tile];
+  if (tid == 0) {
+    const double k = STAGE == 1 ? dt : 0.5 * dt;
+    sm.k = StageK{-k * d.inv_dx, -k * d.inv_dy, 0.0, 0.0, -0.5 * g * k * d.inv_dx,
+                  -0.5 * g * k * d.inv_dy};
+  }
 
   // averages of the tile and its 2-cell halo
-  for (int q = ty * TX + tx; q < HX * HY; q += TX * TY) {
+  for (int q = tid; q < HX * HY; q += TX * TY) {
     const int a = q % HX, b = q / HX;
     const int gi = i0 - 2 + a, gj = j0 - 2 + b;
     double h = 0.0, z = 0.0, qx = 0.0, qy = 0.0;
@@ -162,108 +191,109 @@ __device__ __forceinline__ void fv_tile(const Dev& d, Smem& sm, int bx, int by, 
   __syncthreads();
 
   const int a = tx + 2, b = ty + 2;
-  const bool east_edge = act && (tx == TX - 1 || i == nx - 1);
-  const bool north_edge = act && (ty == TY - 1 || j == ny - 1);
-  L4 E, W, N, S;
-  if (act) {
-    const double(*A)[HY][HX] = sm.u.A;
+  const double(*A)[HY][HX] = sm.u.A;
+  bool b_me = act && every;
+  if (act && !every) {
+    auto moves = [&](int aa, int bb) {
+      return above(A[1][bb][aa], tol) || nonzero(A[2][bb][aa]) || nonzero(A[3][bb][aa]);
+    };
+    b_me = moves(a, b) || moves(a - 1, b) || moves(a + 1, b) || moves(a, b - 1) || moves(a, b + 1);
+  }
+  sm.cls[ty][tx] = (unsigned char)(act ? (b_me ? 2 : 1) : 0);
+  __syncthreads();
+  const bool b_w = tx > 0 && sm.cls[ty][tx - 1] == 2, b_e = tx + 1 < TX && sm.cls[ty][tx + 1] == 2;
+  const bool b_s = ty > 0 && sm.cls[ty - 1][tx] == 2, b_n = ty + 1 < TY && sm.cls[ty + 1][tx] == 2;
+
+  // limits of the computed cells and of their neighbours; the steps of the own free
+  // surface between opposite faces are the slopes of eta
+  L4 W = {}, S = {};
+  double ex = 0.0, ey = 0.0;
+  if (act && (b_me || b_w || b_e || b_s || b_n)) {
     double s[4];
     slopes4<ORDER2>(A, a, b, 1, 0, i == 0 || i == nx - 1, tol, s);
-    E = lim4(A, a, b, s, 0.5);
+    ex = s[0];
+    sm.e[ty][tx] = lim4(A, a, b, s, 0.5);
     W = lim4(A, a, b, s, -0.5);
     slopes4<ORDER2>(A, a, b, 0, 1, j == 0 || j == ny - 1, tol, s);
-    N = lim4(A, a, b, s, 0.5);
+    ey = s[0];
+    sm.n[ty][tx] = lim4(A, a, b, s, 0.5);
     S = lim4(A, a, b, s, -0.5);
-    sm.e[ty][tx] = E;
-    sm.n[ty][tx] = N;
-    if (tx == 0) {
-      if (i == 0) {
-        sm.hw[ty] = ghost4(d, 0, (j + 0.5) * d.dy, ts, W);
-      } else {
-        slopes4<ORDER2>(A, a - 1, b, 1, 0, i - 1 == 0, tol, s);
-        sm.hw[ty] = lim4(A, a - 1, b, s, 0.5);
-      }
-    }
-    if (east_edge) {
-      if (i == nx - 1) {
-        sm.he[ty] = ghost4(d, 1, (j + 0.5) * d.dy, ts, E);
-      } else {
-        slopes4<ORDER2>(A, a + 1, b, 1, 0, i + 1 == nx - 1, tol, s);
-        sm.he[ty] = lim4(A, a + 1, b, s, -0.5);
-      }
-    }
-    if (ty == 0) {
-      if (j == 0) {
-        sm.hs[tx] = ghost4(d, 2, (i + 0.5) * d.dx, ts, S);
-      } else {
-        slopes4<ORDER2>(A, a, b - 1, 0, 1, j - 1 == 0, tol, s);
-        sm.hs[tx] = lim4(A, a, b - 1, s, 0.5);
-      }
-    }
-    if (north_edge) {
-      if (j == ny - 1) {
-        sm.hn[tx] = ghost4(d, 3, (i + 0.5) * d.dx, ts, N);
-      } else {
-        slopes4<ORDER2>(A, a, b + 1, 0, 1, j + 1 == ny - 1, tol, s);
-        sm.hn[tx] = lim4(A, a, b + 1, s, -0.5);
-      }
+  }
+  // the limits beyond the tile, one per thread of the last 2 (TX + TY) threads: west and
+  // east columns, south and north rows, on one code path (as the DG2 stages)
+  const int ni = nx - i0 < TX ? nx - i0 : TX, nj = ny - j0 < TY ? ny - j0 : TY;
+  {
+    const int t = TX * TY - 1 - tid;
+    const int kind = t < TY ? 0 : t < 2 * TY ? 1 : t < 2 * TY + TX ? 2 : 3;
+    const int q = kind == 0 ? t : kind == 1 ? t - TY : kind == 2 ? t - 2 * TY : t - 2 * TY - TX;
+    const int ci = kind == 0 ? 0 : kind == 1 ? ni - 1 : q;
+    const int cj = kind <= 1 ? q : kind == 2 ? 0 : nj - 1;
+    if (t < 2 * (TX + TY) && q < (kind <= 1 ? nj : ni) && sm.cls[cj][ci] == 2) {
+      const int dx = kind <= 1 ? 1 : 0, dy = 1 - dx, side = kind & 1;
+      const int gi = i0 + ci, gj = j0 + cj;
+      const bool at_edge = dx ? (side ? gi == nx - 1 : gi == 0) : (side ? gj == ny - 1 : gj == 0);
+      // the neighbour across the face, or at an edge the tile cell itself
+      const int st = at_edge ? 0 : (side ? 1 : -1);
+      const int la = ci + 2 + dx * st, lb = cj + 2 + dy * st;
+      const int li = gi + dx * st, lj = gj + dy * st;
+      double s[4];
+      slopes4<ORDER2>(A, la, lb, dx, dy, dx ? li == 0 || li == nx - 1 : lj == 0 || lj == ny - 1,
+                      tol, s);
+      L4 r = lim4(A, la, lb, s, (at_edge ? side != 0 : side == 0) ? 0.5 : -0.5);
+      if (at_edge) r = ghost4(d, kind, dx ? (gj + 0.5) * d.dy : (gi + 0.5) * d.dx, ts, r);
+      (kind == 0 ? sm.hw : kind == 1 ? sm.he : kind == 2 ? sm.hs : sm.hn)[q] = r;
     }
   }
   __syncthreads();  // the staged averages are dead past here (the faces reuse them)
 
-  // one revision and one flux per face
-  double dpW = 0.0, dpS = 0.0, dpx;
-  if (act) {
-    const L4& Lw = tx > 0 ? sm.e[ty][tx - 1] : sm.hw[ty];
-    const Face fw = face(Lw, W, false, g, tol, d.flux, dpW);
-    sm.u.f.fx[ty][tx] = fw;
-    if (i == 0) brate += fw.h * d.dy;
-    if (east_edge) {
-      const Face fe = face(E, sm.he[ty], false, g, tol, d.flux, dpx);
-      sm.u.f.fx[ty][tx + 1] = fe;
-      if (i == nx - 1) brate -= fe.h * d.dy;
-    }
-    const L4& Ls = ty > 0 ? sm.n[ty - 1][tx] : sm.hs[tx];
-    const Face fs = face(Ls, S, true, g, tol, d.flux, dpS);
-    sm.u.f.fy[ty][tx] = fs;
-    if (j == 0) brate += fs.h * d.dx;
-    if (north_edge) {
-      const Face fn = face(N, sm.hn[tx], true, g, tol, d.flux, dpx);
-      sm.u.f.fy[ty + 1][tx] = fn;
-      if (j == ny - 1) brate -= fn.h * d.dx;
+  // one revision and one flux per face a computed cell uses: each thread its west and
+  // south faces, then the tile's east and north edge faces one per thread
+  double hW = 0.0, hS = 0.0;  // own revised depths there
+  if (act && (b_me || b_w)) {
+    const Face f = face(tx > 0 ? sm.e[ty][tx - 1] : sm.hw[ty], W, false, g, tol, d.flux, hW);
+    sm.u.f.fx[ty][tx] = f;
+    if (i == 0) brate += f.h * d.dy;
+  }
+  if (act && (b_me || b_s)) {
+    const Face f = face(ty > 0 ? sm.n[ty - 1][tx] : sm.hs[tx], S, true, g, tol, d.flux, hS);
+    sm.u.f.fy[ty][tx] = f;
+    if (j == 0) brate += f.h * d.dx;
+  }
+  {
+    const int t = TX * TY - 1 - tid;
+    const bool yf = t >= TY;
+    const int q = yf ? t - TY : t;
+    if ((yf ? q < ni : q < nj) && (yf ? sm.cls[nj - 1][q] : sm.cls[q][ni - 1]) == 2) {
+      double hb;
+      const Face f = face(yf ? sm.n[nj - 1][q] : sm.e[q][ni - 1], yf ? sm.hn[q] : sm.he[q], yf, g,
+                          tol, d.flux, hb);
+      *(yf ? &sm.u.f.fy[nj][q] : &sm.u.f.fx[q][ni]) = f;
+      if (yf ? j0 + nj == ny : i0 + ni == nx) brate -= f.h * (yf ? d.dx : d.dy);
     }
   }
   __syncthreads();
 
   if (act) {
-    const Face fw = sm.u.f.fx[ty][tx], fe = sm.u.f.fx[ty][tx + 1];
-    const Face fs = sm.u.f.fy[ty][tx], fn = sm.u.f.fy[ty + 1][tx];
-    // own-side bed limits, lowered where the own free surface is below z*
-    const double dE = E.eta - fe.zs, dW = W.eta - fw.zs, dN = N.eta - fn.zs, dS = S.eta - fs.zs;
-    const double zE = fe.zs - (dE < 0.0 ? -dE : 0.0), zW = fw.zs - (dW < 0.0 ? -dW : 0.0);
-    const double zN = fn.zs - (dN < 0.0 ? -dN : 0.0), zS = fs.zs - (dS < 0.0 ? -dS : 0.0);
-    // own pressures and bed term of a direction: g / 2 (hE + hW) times the step of the
-    // free surface between the faces
-    const double bx = 0.5 * g * (fe.ha + fw.hb) * ((fe.ha - fw.hb) + (zE - zW));
-    const double by = 0.5 * g * (fn.ha + fs.hb) * ((fn.ha - fs.hb) + (zN - zS));
-    const double idx = d.inv_dx, idy = d.inv_dy;
-    // Eq. 8
-    double Lh = -(fe.h - fw.h) * idx - (fn.h - fs.h) * idy;
-    const double Lx = -((fe.n - (fw.n + dpW)) + bx) * idx - (fn.t - fs.t) * idy;
-    const double Ly = -(fe.t - fw.t) * idx - ((fn.n - (fs.n + dpS)) + by) * idy;
-    if (d.rain != 0.0 && ts >= d.rain_t0 && ts < d.rain_t1) Lh += d.rain;
-    if (c == d.src_idx) Lh += d.qp * idx * idy;
-    double h, qx, qy;
-    if (STAGE == 1) {
-      h = d.S[H0 * P + c] + dt * Lh;
-      qx = d.S[QX0 * P + c] + dt * Lx;
-      qy = d.S[QY0 * P + c] + dt * Ly;
-    } else {
-      h = 0.5 * (d.S[H0 * P + c] + d.T[H0 * P + c] + dt * Lh);
-      qx = 0.5 * (d.S[QX0 * P + c] + d.T[QX0 * P + c] + dt * Lx);
-      qy = 0.5 * (d.S[QY0 * P + c] + d.T[QY0 * P + c] + dt * Ly);
+    double h = d.S[H0 * P + c], qx = d.S[QX0 * P + c], qy = d.S[QY0 * P + c];
+    if (STAGE == 2) {
+      h = half64(h + d.T[H0 * P + c]);
+      qx = half64(qx + d.T[QX0 * P + c]);
+      qy = half64(qy + d.T[QY0 * P + c]);
     }
-    if (h <= tol) { qx = 0.0; qy = 0.0; }
+    if (b_me) {
+      // Eq. 8 with the own pressures in the bed terms: g / 2 (hE + hW) times the step of
+      // the own free surface between the faces (see Flux)
+      const StageK K = sm.k;
+      const Face &fw = sm.u.f.fx[ty][tx], &fe = sm.u.f.fx[ty][tx + 1];
+      const Face &fs = sm.u.f.fy[ty][tx], &fn = sm.u.f.fy[ty + 1][tx];
+      h += fma(K.dx, fe.h - fw.h, K.dy * (fn.h - fs.h));
+      qx += fma(K.dx, fe.n - (fw.n + fw.dp), fma(K.dy, fn.t - fs.t, K.bx * ex * (fe.ha + hW)));
+      qy += fma(K.dx, fe.t - fw.t, fma(K.dy, fn.n - (fs.n + fs.dp), K.by * ey * (fn.ha + hS)));
+      const double k = STAGE == 1 ? dt : 0.5 * dt;
+      if (d.rain != 0.0 && ts >= d.rain_t0 && ts < d.rain_t1) h += k * d.rain;
+      if (c == d.src_idx) h += k * (d.qp * d.inv_dx * d.inv_dy);
+    }
+    if (!above(h, tol)) { qx = 0.0; qy = 0.0; }
     double* O = STAGE == 1 ? d.T : d.S;
     O[H0 * P + c] = h;
     O[QX0 * P + c] = qx;
@@ -271,7 +301,7 @@ __device__ __forceinline__ void fv_tile(const Dev& d, Smem& sm, int bx, int by, 
     if (STAGE == 2 || !ORDER2) {
       lam = cell_rate(d, h, qx, qy);
       bad = bad || !(isfinite(h) && isfinite(qx) && isfinite(qy)) || h < -1.0;
-      nonq = !(h <= tol) || qx != 0.0 || qy != 0.0;
+      nonq = above(h, tol) || nonzero(qx) || nonzero(qy);
     }
   }
 }
