@@ -52,10 +52,7 @@ namespace DG2_ADJ_NS {
 // is compiled once for each).  Kernels load stored values into FP64 registers and
 // round their results to the storage type; the hydrograph, the step times, the
 // per-step discharge adjoint sums and the misfit stay FP64.
-#ifndef DG2_ADJ_ARITH
-#define DG2_ADJ_ARITH double
-#endif
-using real = DG2_ADJ_ARITH;
+using real = double;
 using store = DG2_ADJ_STORE;
 
 // ---------------------------------------------------------------------------
@@ -175,6 +172,47 @@ template <class T>
 __device__ __forceinline__ T tmin(const T& a, const T& b) { return val(b) < val(a) ? b : a; }
 template <class T>
 __device__ __forceinline__ T tmax(const T& a, const T& b) { return val(b) > val(a) ? b : a; }
+
+// Reciprocal, square root and h^(-7/3) of the reverse sweeps: the solver's short FP64 forms
+// on the device, the plain ones where these functions are compiled for the host.
+__device__ __forceinline__ double recip(double x) {
+#ifdef __CUDA_ARCH__
+  return rcp64(x);
+#else
+  return 1.0 / x;
+#endif
+}
+__device__ __forceinline__ double root(double x) {
+#ifdef __CUDA_ARCH__
+  return sqrt64(x);
+#else
+  return ::sqrt(x);
+#endif
+}
+__device__ __forceinline__ double inv_pow73(double h) {
+#ifdef __CUDA_ARCH__
+  return h_m73(h);
+#else
+  return 1.0 / (h * h * ::cbrt(h));
+#endif
+}
+// (u, v) = (qx, qy) / h
+__device__ __forceinline__ void velocity(double qx, double qy, double h, double& u, double& v) {
+#ifdef DG2_ADJ_STORE32
+  u = qx / h;  // the FP32 forward's arithmetic is kept as measured (fwd_stage_kernel)
+  v = qy / h;
+#else
+  const double ih = recip(h);
+  u = qx * ih;
+  v = qy * ih;
+#endif
+}
+template <int N>
+__device__ __forceinline__ void velocity(const Dual<N>& qx, const Dual<N>& qy, const Dual<N>& h,
+                                         Dual<N>& u, Dual<N>& v) {
+  u = qx / h;
+  v = qy / h;
+}
 
 // ---------------------------------------------------------------------------
 // The scheme's point functions, templated on the scalar (real or Dual)
@@ -345,8 +383,7 @@ __device__ __forceinline__ RecT<T> make_rec_t(const T& h, const T& qx, const T& 
     r.u = 2.0 * hp * qx / den;
     r.v = 2.0 * hp * qy / den;
   } else if (val(h) > tol) {
-    r.u = qx / h;
-    r.v = qy / h;
+    velocity(qx, qy, h, r.u, r.v);
   }
   const T hp = pos_t(h);
   r.hs = pw ? sc * hp : hp;
@@ -431,7 +468,7 @@ __device__ __noinline__ void revise_flux_adj(const RecT<real>& a, const RecT<rea
   real g_hR = 0.0, g_qnR = 0.0, g_qtR = 0.0, g_unR = 0.0, g_utR = 0.0;
   if (!(hL <= tol && hR <= tol)) {
     // ---- forward: HLL (hll_t) ----
-    const real cL = sqrt(gr * hL), cR = sqrt(gr * hR);
+    const real cL = root(gr * hL), cR = root(gr * hR);
     real sL, sR, us = 0.0, cs = 0.0;
     int mode;
     bool sL_first = true, sR_first = true;
@@ -463,7 +500,7 @@ __device__ __noinline__ void revise_flux_adj(const RecT<real>& a, const RecT<rea
       for (int k = 0; k < 3; ++k) g_fR[k] = w[k];
     } else {
       // F_k = (sR fL_k - sL fR_k + sL sR (qR_k - qL_k)) / (sR - sL)
-      const real inv = 1.0 / (sR - sL), sLR = sL * sR;
+      const real inv = recip(sR - sL), sLR = sL * sR;
       const real dq[3] = {hR - hL, qnR - qnL, qtR - qtL};
       real g_sL = 0.0, g_sR = 0.0, g_inv = 0.0, g_dq[3];
       for (int k = 0; k < 3; ++k) {
@@ -499,8 +536,8 @@ __device__ __noinline__ void revise_flux_adj(const RecT<real>& a, const RecT<rea
         g_cR += -g_us + 0.5 * g_cs;
       }
       // c = sqrt(g h): dc/dh = g / (2 c), 0 at c = 0
-      if (cL > 0.0) g_hL += g_cL * (0.5 * gr / cL);
-      if (cR > 0.0) g_hR += g_cR * (0.5 * gr / cR);
+      if (cL > 0.0) g_hL += g_cL * (0.5 * gr * recip(cL));
+      if (cR > 0.0) g_hR += g_cR * (0.5 * gr * recip(cR));
     }
     // physical fluxes f = (h un, h un^2 + g h^2 / 2, h un ut)
     g_hL += g_fL[0] * unL + g_fL[1] * (unL * unL + gr * hL) + g_fL[2] * unL * utL;
@@ -661,7 +698,7 @@ __device__ __forceinline__ void own_terms(const Prob& p, const T* hs, const T* z
 __device__ __forceinline__ void phys_adj(real h, real qx, real qy, real gr, real tol, bool ydir,
                                          const real* gf, real& g_h, real& g_qx, real& g_qy) {
   const bool wet = h > tol;
-  const real u = wet ? qx / h : 0.0, v = wet ? qy / h : 0.0;
+  const real ih = wet ? recip(h) : 0.0, u = qx * ih, v = qy * ih;
   real gh, gu, gv;
   if (!ydir) {  // (h u, h u^2 + g h^2 / 2, h u v)
     gh = gf[0] * u + gf[1] * (u * u + gr * h) + gf[2] * u * v;
@@ -673,9 +710,9 @@ __device__ __forceinline__ void phys_adj(real h, real qx, real qy, real gr, real
     gv = gf[0] * h + gf[1] * h * u + gf[2] * 2.0 * h * v;
   }
   if (wet) {  // u = qx / h, v = qy / h
-    g_qx += gu / h;
-    g_qy += gv / h;
-    gh -= (gu * u + gv * v) / h;
+    g_qx += gu * ih;
+    g_qy += gv * ih;
+    gh -= (gu * u + gv * v) * ih;
   }
   g_h += gh;
 }
@@ -804,10 +841,10 @@ __device__ __forceinline__ void rec_uv_adj(real h, real qx, real qy, bool thin, 
     g_h += g_den * 2.0 * h;
     g_h0 += g_den * 2.0 * eps * 0.1;
   } else if (h > tol) {
-    const real u = qx / h, v = qy / h;
-    g_qx += gu / h;
-    g_qy += gv / h;
-    g_h -= (gu * u + gv * v) / h;
+    const real ih = recip(h), u = qx * ih, v = qy * ih;
+    g_qx += gu * ih;
+    g_qy += gv * ih;
+    g_h -= (gu * u + gv * v) * ih;
   }
 }
 
@@ -850,6 +887,163 @@ __device__ __noinline__ void side_rec_adj(const Prob& p, const real* h4, real qx
   g[5] = g_qy;
 }
 
+// Friction of one cell (Sec. 2.1.3): modes m -> out, the function that friction_cell_adj
+// differentiates (the forward kernel works on the solver's own point update).
+template <class T>
+__device__ __forceinline__ void friction_point_t(const T& gn2dt, real tol, const T& h, T& qx,
+                                                 T& qy) {
+  if (!(val(h) > tol)) return;
+  const T qm = sqrt(qx * qx + qy * qy);
+  const T den = 1.0 + gn2dt * qm / (h * h * cbrt(h));
+  qx = qx / den;
+  qy = qy / den;
+}
+
+template <class T>
+__device__ __forceinline__ void friction_cell(const T* m, const T& n, real dt, real g, real tol,
+                                              T* out) {
+#pragma unroll
+  for (int k = 0; k < 9; ++k) out[k] = m[k];
+  const T gn2dt = dt * g * n * n;
+  T cx = m[QX0], cy = m[QY0];
+  friction_point_t(gn2dt, tol, m[H0], cx, cy);
+  const real r3 = 1.0 / 1.7320508075688772, hs3 = 0.5 * 1.7320508075688772;
+#pragma unroll
+  for (int dd = 1; dd <= 2; ++dd) {
+    const T h1 = m[dd], x1 = m[3 + dd], y1 = m[6 + dd];
+    T xp = m[QX0] + x1 * r3, yp = m[QY0] + y1 * r3, xm = m[QX0] - x1 * r3, ym = m[QY0] - y1 * r3;
+    friction_point_t(gn2dt, tol, m[H0] + h1 * r3, xp, yp);
+    friction_point_t(gn2dt, tol, m[H0] - h1 * r3, xm, ym);
+    out[3 + dd] = hs3 * (xp - xm);
+    out[6 + dd] = hs3 * (yp - ym);
+  }
+  out[QX0] = cx;
+  out[QY0] = cy;
+}
+
+// Reverse-mode adjoint of one friction point (q /= 1 + gn2dt |q| h^(-7/3)): given the
+// adjoints (wx, wy) of the updated discharges, adds the gradient into g_gn2dt,
+// g_h, g_qx, g_qy (a dry point is the identity).  One reciprocal per denominator and
+// h^(-7/3) by its series: some 45 FP64 instructions, about 200 with a cube root and eight
+// divisions (adj_cell_kernel<1>, which is mostly this: 674 -> 180 us at 512 x 512).
+__device__ __forceinline__ void friction_point_adj(real gn2dt, real tol, real h, real qx, real qy,
+                                                   real wx, real wy, real& g_gn2dt, real& g_h,
+                                                   real& g_qx, real& g_qy) {
+  if (!(h > tol)) {
+    g_qx += wx;
+    g_qy += wy;
+    return;
+  }
+  const real qm = root(qx * qx + qy * qy);
+  const real s = inv_pow73(h);
+  const real den = 1.0 + gn2dt * qm * s;
+  const real iden = den < 1e300 ? recip(den) : 0.0;
+  g_qx += wx * iden;
+  g_qy += wy * iden;
+  // d(q / den) = -q / den^2 per unit of den, den = 1 + gn2dt |q| s
+  const real gs = -(wx * qx + wy * qy) * (iden * iden) * s, gsq = gs * qm;
+  g_gn2dt += gsq;
+  g_h += gsq * gn2dt * (-7.0 / 3.0) * recip(h);  // ds/dh = -7/3 s / h
+  if (qm > 0.0) {
+    const real g_qm = gs * gn2dt * recip(qm);
+    g_qx += g_qm * qx;
+    g_qy += g_qm * qy;
+  }
+}
+
+// Reverse-mode adjoint of friction_cell: the gradient of ls . Fric(m; n) with
+// respect to the modes m (g_m) and the Manning n (g_n).
+__device__ __noinline__ void friction_cell_adj(const real* m, real n, real dt, real g, real tol,
+                                               const real* ls, real* g_m, real& g_n) {
+  const real gn2dt = dt * g * n * n;
+  real g_gn2dt = 0.0;
+  for (int k = 0; k < 9; ++k) g_m[k] = 0.0;
+  // depth modes pass through
+  g_m[H0] += ls[H0];
+  g_m[H1X] += ls[H1X];
+  g_m[H1Y] += ls[H1Y];
+  // centre
+  friction_point_adj(gn2dt, tol, m[H0], m[QX0], m[QY0], ls[QX0], ls[QY0], g_gn2dt, g_m[H0],
+                     g_m[QX0], g_m[QY0]);
+  const real r3 = 1.0 / 1.7320508075688772, hs3 = 0.5 * 1.7320508075688772;
+  for (int dd = 1; dd <= 2; ++dd) {
+    // out[3 + dd] = hs3 (xp - xm), out[6 + dd] = hs3 (yp - ym)
+    const real wx = hs3 * ls[3 + dd], wy = hs3 * ls[6 + dd];
+    const real h1 = m[dd], x1 = m[3 + dd], y1 = m[6 + dd];
+    for (int sgn = 0; sgn < 2; ++sgn) {
+      const real r = sgn == 0 ? r3 : -r3, w = sgn == 0 ? 1.0 : -1.0;
+      real gh = 0.0, gx = 0.0, gy = 0.0;
+      friction_point_adj(gn2dt, tol, m[H0] + h1 * r, m[QX0] + x1 * r, m[QY0] + y1 * r, w * wx,
+                         w * wy, g_gn2dt, gh, gx, gy);
+      g_m[H0] += gh;
+      g_m[dd] += gh * r;
+      g_m[QX0] += gx;
+      g_m[3 + dd] += gx * r;
+      g_m[QY0] += gy;
+      g_m[6 + dd] += gy * r;
+    }
+  }
+  // gn2dt = dt g n^2
+  g_n = g_gn2dt * 2.0 * dt * g * n;
+}
+
+// ---------------------------------------------------------------------------
+// Forward kernels (one thread per cell, dense planes)
+// ---------------------------------------------------------------------------
+
+// Wet-dry treatment after a stage (mass-neutral); returns the 9-bit mask of
+// the modes it keeps.
+__device__ __forceinline__ unsigned wetdry_mask(double* m, double z0, double z1x, double z1y,
+                                                double tol) {
+  const double h0 = m[H0];
+  if (!above(h0, tol)) {
+#pragma unroll
+    for (int k = 1; k < 9; ++k) m[k] = 0.0;
+    return 1u;
+  }
+  unsigned keep = 0x1FFu;
+  const bool de = !above(h0 + m[H1X], tol), dw = !above(h0 - m[H1X], tol);
+  const bool dn = !above(h0 + m[H1Y], tol), ds = !above(h0 - m[H1Y], tol);
+  if (de || dw || dn || ds) {
+    const double eta0 = h0 + z0;
+    if ((de && !gt(z0 + z1x, eta0)) || (dw && !gt(z0 - z1x, eta0))) {
+      m[H1X] = 0.0; m[QX1X] = 0.0; m[QY1X] = 0.0;
+      keep &= ~((1u << H1X) | (1u << QX1X) | (1u << QY1X));
+    }
+    if ((dn && !gt(z0 + z1y, eta0)) || (ds && !gt(z0 - z1y, eta0))) {
+      m[H1Y] = 0.0; m[QX1Y] = 0.0; m[QY1Y] = 0.0;
+      keep &= ~((1u << H1Y) | (1u << QX1Y) | (1u << QY1Y));
+    }
+  }
+  return keep;
+}
+
+// Friction of one cell (Sec. 2.1.3): the forward solver's point update at the centre and
+// the Gauss points, in place.
+__device__ __forceinline__ void friction_forward(double* m, double n, double dt, double g,
+                                              double tol) {
+  const double gn2dt = dt * g * n * n;
+  const double r3 = 1.0 / 1.7320508075688772, hs3 = 0.5 * 1.7320508075688772;
+  const double x0 = m[QX0], y0 = m[QY0];
+  friction_point(gn2dt, tol, m[H0], m[QX0], m[QY0]);
+#pragma unroll
+  for (int dd = 1; dd <= 2; ++dd) {
+    const double h1 = m[dd], x1 = m[3 + dd], y1 = m[6 + dd];
+    double xp = x0 + x1 * r3, yp = y0 + y1 * r3, xm = x0 - x1 * r3, ym = y0 - y1 * r3;
+    friction_point(gn2dt, tol, m[H0] + h1 * r3, xp, yp);
+    friction_point(gn2dt, tol, m[H0] - h1 * r3, xm, ym);
+    m[3 + dd] = hs3 * (xp - xm);
+    m[6 + dd] = hs3 * (yp - ym);
+  }
+}
+
+#ifdef DG2_ADJ_STORE32
+// FP32 storage: one thread per cell, each building its four faces, with the templated point
+// functions above.  The tiled kernel below is no less exact, but a stored FP32 state rounds
+// differently under any other arithmetic, and the calibration trajectories grow round-off
+// tenfold in 300 steps: on the 16 x 16 window the FP32 misfit's error is 0.037 this way and
+// 0.15 with the tiled kernel, where 48 runs of either with step sizes changed by 1e-12 gave
+// 0.0005 to 0.38.  The stated error stays the one that was measured.
 // Face on side f (0 E, 1 W, 2 N, 3 S) of cell (i, j) of state U at stage time
 // with hydrograph discharge Q, in real: its flux and the own side's revised
 // depth and bed level.
@@ -929,138 +1123,6 @@ __device__ void cell_operator(const Prob& p, const store* __restrict__ U, int i,
   if (p.rain != 0.0 && t >= p.rain_t0 && t < p.rain_t1) L[H0] += p.rain;
 }
 
-// Wet-dry treatment after a stage (mass-neutral); returns the 9-bit mask of
-// the modes it keeps.
-__device__ __forceinline__ unsigned wetdry_mask(real* m, real z0, real z1x, real z1y,
-                                                real tol) {
-  const real h0 = m[H0];
-  if (h0 <= tol) {
-#pragma unroll
-    for (int k = 1; k < 9; ++k) m[k] = 0.0;
-    return 1u;
-  }
-  unsigned keep = 0x1FFu;
-  const real eta0 = h0 + z0;
-  {
-    const bool fe = (h0 + m[H1X] <= tol) && !(z0 + z1x > eta0);
-    const bool fw = (h0 - m[H1X] <= tol) && !(z0 - z1x > eta0);
-    if (fe || fw) {
-      m[H1X] = 0.0; m[QX1X] = 0.0; m[QY1X] = 0.0;
-      keep &= ~((1u << H1X) | (1u << QX1X) | (1u << QY1X));
-    }
-  }
-  {
-    const bool fn = (h0 + m[H1Y] <= tol) && !(z0 + z1y > eta0);
-    const bool fs = (h0 - m[H1Y] <= tol) && !(z0 - z1y > eta0);
-    if (fn || fs) {
-      m[H1Y] = 0.0; m[QX1Y] = 0.0; m[QY1Y] = 0.0;
-      keep &= ~((1u << H1Y) | (1u << QX1Y) | (1u << QY1Y));
-    }
-  }
-  return keep;
-}
-
-// Friction of one cell (Sec. 2.1.3, as the forward solver): modes m -> out.
-template <class T>
-__device__ __forceinline__ void friction_point_t(const T& gn2dt, real tol, const T& h, T& qx,
-                                                 T& qy) {
-  if (!(val(h) > tol)) return;
-  const T qm = sqrt(qx * qx + qy * qy);
-  const T den = 1.0 + gn2dt * qm / (h * h * cbrt(h));
-  qx = qx / den;
-  qy = qy / den;
-}
-
-template <class T>
-__device__ __forceinline__ void friction_cell(const T* m, const T& n, real dt, real g, real tol,
-                                              T* out) {
-#pragma unroll
-  for (int k = 0; k < 9; ++k) out[k] = m[k];
-  const T gn2dt = dt * g * n * n;
-  T cx = m[QX0], cy = m[QY0];
-  friction_point_t(gn2dt, tol, m[H0], cx, cy);
-  const real r3 = 1.0 / 1.7320508075688772, hs3 = 0.5 * 1.7320508075688772;
-#pragma unroll
-  for (int dd = 1; dd <= 2; ++dd) {
-    const T h1 = m[dd], x1 = m[3 + dd], y1 = m[6 + dd];
-    T xp = m[QX0] + x1 * r3, yp = m[QY0] + y1 * r3, xm = m[QX0] - x1 * r3, ym = m[QY0] - y1 * r3;
-    friction_point_t(gn2dt, tol, m[H0] + h1 * r3, xp, yp);
-    friction_point_t(gn2dt, tol, m[H0] - h1 * r3, xm, ym);
-    out[3 + dd] = hs3 * (xp - xm);
-    out[6 + dd] = hs3 * (yp - ym);
-  }
-  out[QX0] = cx;
-  out[QY0] = cy;
-}
-
-// Reverse-mode adjoint of one friction point (friction_point_t): given the
-// adjoints (wx, wy) of the updated discharges, adds the gradient into g_gn2dt,
-// g_h, g_qx, g_qy (a dry point is the identity).
-__device__ __forceinline__ void friction_point_adj(real gn2dt, real tol, real h, real qx, real qy,
-                                                   real wx, real wy, real& g_gn2dt, real& g_h,
-                                                   real& g_qx, real& g_qy) {
-  if (!(h > tol)) {
-    g_qx += wx;
-    g_qy += wy;
-    return;
-  }
-  const real qm = sqrt(qx * qx + qy * qy);
-  const real D = h * h * cbrt(h);  // h^(7/3)
-  const real den = 1.0 + gn2dt * qm / D;
-  const real ox = qx / den, oy = qy / den;
-  g_qx += wx / den;
-  g_qy += wy / den;
-  const real g_den = -(wx * ox + wy * oy) / den;
-  g_gn2dt += g_den * qm / D;
-  const real g_qm = g_den * gn2dt / D;
-  const real g_D = -g_den * gn2dt * qm / (D * D);
-  g_h += g_D * (7.0 / 3.0) * D / h;
-  if (qm > 0.0) {
-    g_qx += g_qm * qx / qm;
-    g_qy += g_qm * qy / qm;
-  }
-}
-
-// Reverse-mode adjoint of friction_cell: the gradient of ls . Fric(m; n) with
-// respect to the modes m (g_m) and the Manning n (g_n).
-__device__ __noinline__ void friction_cell_adj(const real* m, real n, real dt, real g, real tol,
-                                               const real* ls, real* g_m, real& g_n) {
-  const real gn2dt = dt * g * n * n;
-  real g_gn2dt = 0.0;
-  for (int k = 0; k < 9; ++k) g_m[k] = 0.0;
-  // depth modes pass through
-  g_m[H0] += ls[H0];
-  g_m[H1X] += ls[H1X];
-  g_m[H1Y] += ls[H1Y];
-  // centre
-  friction_point_adj(gn2dt, tol, m[H0], m[QX0], m[QY0], ls[QX0], ls[QY0], g_gn2dt, g_m[H0],
-                     g_m[QX0], g_m[QY0]);
-  const real r3 = 1.0 / 1.7320508075688772, hs3 = 0.5 * 1.7320508075688772;
-  for (int dd = 1; dd <= 2; ++dd) {
-    // out[3 + dd] = hs3 (xp - xm), out[6 + dd] = hs3 (yp - ym)
-    const real wx = hs3 * ls[3 + dd], wy = hs3 * ls[6 + dd];
-    const real h1 = m[dd], x1 = m[3 + dd], y1 = m[6 + dd];
-    for (int sgn = 0; sgn < 2; ++sgn) {
-      const real r = sgn == 0 ? r3 : -r3, w = sgn == 0 ? 1.0 : -1.0;
-      real gh = 0.0, gx = 0.0, gy = 0.0;
-      friction_point_adj(gn2dt, tol, m[H0] + h1 * r, m[QX0] + x1 * r, m[QY0] + y1 * r, w * wx,
-                         w * wy, g_gn2dt, gh, gx, gy);
-      g_m[H0] += gh;
-      g_m[dd] += gh * r;
-      g_m[QX0] += gx;
-      g_m[3 + dd] += gx * r;
-      g_m[QY0] += gy;
-      g_m[6 + dd] += gy * r;
-    }
-  }
-  // gn2dt = dt g n^2
-  g_n = g_gn2dt * 2.0 * dt * g * n;
-}
-
-// ---------------------------------------------------------------------------
-// Forward kernels (one thread per cell, dense planes)
-// ---------------------------------------------------------------------------
-
 __global__ void fwd_friction_kernel(Prob p, const store* __restrict__ U, store* __restrict__ Us,
                                     real dt) {
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1093,6 +1155,151 @@ __global__ void fwd_stage_kernel(Prob p, const store* __restrict__ Us, const sto
 #pragma unroll
   for (int k = 0; k < 9; ++k) Uo[k * p.N + c] = o[k];
 }
+
+#else
+__global__ void __launch_bounds__(256) fwd_friction_kernel(Prob p, const store* __restrict__ U,
+                                                           store* __restrict__ Us, real dt) {
+  const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= p.N) return;
+  double m[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) m[k] = U[k * p.N + c];
+  friction_forward(m, p.Nm[c], dt, p.g, p.tol);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) Us[k * p.N + c] = m[k];
+}
+
+// Stage 1: U1 = W(Us + dt L(Us, t)); stage 2: Uo = W((Us + U1 + dt L(U1, t)) / 2), on
+// tiles of AX x AY cells, one thread each, with the FP64 solver's records, faces and update
+// (dg2_device.cuh): every record is built and every face revised and fluxed once per tile.
+// The FP64 pipe bounds it.  One thread per cell without tiles built each record twice and
+// each face twice, with full divisions and roots: 434 / 442 us a launch at 512 x 512 cells
+// then, 146 / 161 us now (friction 146 -> 69 us).  16 x 8 rather than 32 x 8 cells: the calibration grids are small, and a tile's arithmetic is long
+// enough that whole SMs would idle in the last wave.  rev (may be null) takes the revised
+// depth and bed of each face (planes 2f, 2f + 1 of faces E, W, N, S), which the reverse
+// sweep's own-terms pass reads.
+constexpr int AX = 16, AY = 8;
+struct FwdSmem {
+  Rec e[AY][AX], n[AY][AX];              // east / north record of each cell
+  Rec hw[AY], he[AY], hs[AX], hn[AX];    // records beyond the tile
+  FaceR fx[AY][AX + 1], fy[AY + 1][AX];  // west / south face of each cell, edges last
+  StageK k;
+};
+
+template <int STAGE>
+__global__ void __launch_bounds__(AX* AY, 4)
+    fwd_stage_kernel(Prob p, const store* __restrict__ Us, const store* __restrict__ U1,
+                     store* __restrict__ Uo, unsigned short* __restrict__ mask, double dt, double t,
+                     double Q, store* __restrict__ rev) {
+  __shared__ FwdSmem sm;
+  const int tid = threadIdx.x, tx = tid % AX, ty = tid / AX;
+  const int i0 = blockIdx.x * AX, j0 = blockIdx.y * AY, i = i0 + tx, j = j0 + ty;
+  const bool act = i < p.nx && j < p.ny;
+  const long long N = p.N, c = (long long)j * p.nx + i;
+  const store* __restrict__ In = STAGE == 1 ? Us : U1;
+  const double g = p.g, tol = p.tol, kt = STAGE == 1 ? dt : 0.5 * dt;
+  if (tid == 0)
+    sm.k = StageK{-kt * p.inv_dx, -kt * p.inv_dy, -3.0 * kt * p.inv_dx, -3.0 * kt * p.inv_dy,
+                  -0.5 * g * kt * p.inv_dx, -0.5 * g * kt * p.inv_dy};
+  double m[9], z0 = 0.0, z1x = 0.0, z1y = 0.0;
+  Rec rW, rS;
+  if (act) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) m[k] = In[k * N + c];
+    z0 = p.Z[c];
+    z1x = p.Z[N + c];
+    z1y = p.Z[2 * N + c];
+    const double eh = m[H0] + m[H1X], wh = m[H0] - m[H1X];
+    const double nh = m[H0] + m[H1Y], sh = m[H0] - m[H1Y];
+    double scl;
+    const bool pw = pw_scale(m[H0], wh, eh, sh, nh, tol, p.wd, scl), thin = p.wd != 0;
+    sm.e[ty][tx] = make_rec(eh, m[QX0] + m[QX1X], m[QY0] + m[QY1X], z0 + z1x, pw, scl, tol, thin, m[H0]);
+    rW = make_rec(wh, m[QX0] - m[QX1X], m[QY0] - m[QY1X], z0 - z1x, pw, scl, tol, thin, m[H0]);
+    sm.n[ty][tx] = make_rec(nh, m[QX0] + m[QX1Y], m[QY0] + m[QY1Y], z0 + z1y, pw, scl, tol, thin, m[H0]);
+    rS = make_rec(sh, m[QX0] - m[QX1Y], m[QY0] - m[QY1Y], z0 - z1y, pw, scl, tol, thin, m[H0]);
+  }
+  // records beyond the tile: a neighbour's, or the ghost of the tile cell's own limit
+  const int ni = p.nx - i0 < AX ? p.nx - i0 : AX, nj = p.ny - j0 < AY ? p.ny - j0 : AY;
+  {
+    const int kind = tid < AY ? 0 : tid < 2 * AY ? 1 : tid < 2 * AY + AX ? 2 : 3;
+    const int q = kind == 0 ? tid : kind == 1 ? tid - AY : kind == 2 ? tid - 2 * AY : tid - 2 * AY - AX;
+    if (tid < 2 * (AX + AY) && q < (kind <= 1 ? nj : ni)) {
+      const int gi = i0 + (kind == 0 ? 0 : kind == 1 ? ni - 1 : q);
+      const int gj = j0 + (kind <= 1 ? q : kind == 2 ? 0 : nj - 1);
+      const int dir = kind <= 1 ? 1 : 2, side = kind & 1;
+      const bool at_edge = dir == 1 ? (side == 0 ? gi == 0 : gi == p.nx - 1)
+                                    : (side == 0 ? gj == 0 : gj == p.ny - 1);
+      const int step = at_edge ? 0 : (side == 0 ? -1 : 1);
+      const long long cc = (long long)(gj + (dir == 2 ? step : 0)) * p.nx + gi + (dir == 1 ? step : 0);
+      // the limit at the shared face: of the neighbour's near side, or the own cell's
+      const double sg = (side == 0) != at_edge ? 1.0 : -1.0;
+      const double h0 = In[cc], hx = In[H1X * N + cc], hy = In[H1Y * N + cc];
+      double h = h0 + sg * (dir == 1 ? hx : hy);
+      double qx = In[QX0 * N + cc] + sg * In[(QX0 + dir) * N + cc];
+      double qy = In[QY0 * N + cc] + sg * In[(QY0 + dir) * N + cc];
+      const double zf = p.Z[cc] + sg * p.Z[dir * N + cc];
+      Rec r;
+      if (at_edge) {
+        ghost_t<double>(p, kind, dir == 1 ? (gj + 0.5) * p.dy : (gi + 0.5) * p.dx, Q, h, qx, qy);
+        r = make_rec(h, qx, qy, zf, false, 1.0, tol);
+      } else {
+        double scl;
+        const bool pw = pw_scale(h0, h0 - hx, h0 + hx, h0 - hy, h0 + hy, tol, p.wd, scl);
+        r = make_rec(h, qx, qy, zf, pw, scl, tol, p.wd != 0, h0);
+      }
+      (kind == 0 ? sm.hw : kind == 1 ? sm.he : kind == 2 ? sm.hs : sm.hn)[q] = r;
+    }
+  }
+  __syncthreads();
+
+  Side W = {}, S = {};          // the own side of the west and south faces
+  double dpW = 0.0, dpS = 0.0;  // their pressure steps
+  if (act) {
+    FaceR f;
+    Flux w = revise_face<false>(tx > 0 ? sm.e[ty][tx - 1] : sm.hw[ty], rW, false, g, tol, f.a, W);
+    f.h = w.h; f.n = w.n; f.t = w.t;
+    sm.fx[ty][tx] = f;
+    dpW = w.dp;
+    w = revise_face<false>(ty > 0 ? sm.n[ty - 1][tx] : sm.hs[tx], rS, true, g, tol, f.a, S);
+    f.h = w.h; f.n = w.n; f.t = w.t;
+    sm.fy[ty][tx] = f;
+    dpS = w.dp;
+  }
+  {
+    const bool yf = tid >= AY;
+    const int q = yf ? tid - AY : tid;
+    if (yf ? q < ni : q < nj) {
+      FaceR f;
+      Side b;
+      const Flux w = revise_face<false>(yf ? sm.n[nj - 1][q] : sm.e[q][ni - 1],
+                                        yf ? sm.hn[q] : sm.he[q], yf, g, tol, f.a, b);
+      f.h = w.h; f.n = w.n; f.t = w.t;
+      *(yf ? &sm.fy[nj][q] : &sm.fx[q][ni]) = f;
+    }
+  }
+  __syncthreads();
+  if (!act) return;
+
+  double out[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k)
+    out[k] = STAGE == 1 ? m[k] : half64(Us[k * N + c] + m[k]);
+  const Side E = sm.fx[ty][tx + 1].a, Nn = sm.fy[ty + 1][tx].a;
+  if (rev) {
+    rev[0 * N + c] = E.h;  rev[1 * N + c] = E.z;
+    rev[2 * N + c] = W.h;  rev[3 * N + c] = W.z;
+    rev[4 * N + c] = Nn.h; rev[5 * N + c] = Nn.z;
+    rev[6 * N + c] = S.h;  rev[7 * N + c] = S.z;
+  }
+  apply_operator(sm.k, sm.fx[ty][tx], sm.fx[ty][tx + 1], W, dpW, sm.fy[ty][tx], sm.fy[ty + 1][tx], S,
+                 dpS, tol, out);
+  if (p.rain != 0.0 && t >= p.rain_t0 && t < p.rain_t1) out[H0] += kt * p.rain;
+  mask[c] = (unsigned short)wetdry_mask(out, z0, z1x, z1y, tol);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) Uo[k * N + c] = out[k];
+}
+
+#endif
 
 // Sampled gauge depths max(0, planar h) of state U.
 __global__ void gauge_kernel(const store* __restrict__ U, long long N, int ng,
@@ -1587,34 +1794,37 @@ int launch_ok() {
 unsigned blocks(long long n) { return (unsigned)((n + 255) / 256); }
 
 // One forward step k from Uin to Uout (Us, U1, masks left in the workspace;
-// with keep_rev also each stage's revised face depths and beds).
+// with keep_rev also each stage's revised face depths and beds).  Uout may be Uin, which
+// only the friction reads.
 int fwd_step(Ctx* a, int k, double t, const store* Uin, store* Uout, bool keep_rev = false) {
   const double dt = a->dts[k];
   store* Us = dptr(a, a->lay.off_Us);
   store* U1 = dptr(a, a->lay.off_U1);
   unsigned short* m1 = (unsigned short*)(a->ws + a->lay.off_m1);
   unsigned short* m2 = (unsigned short*)(a->ws + a->lay.off_m2);
-  const unsigned nb = blocks(a->lay.N);
-  fwd_friction_kernel<<<nb, 256, 0, a->st>>>(a->p, Uin, Us, dt);
+#ifdef DG2_ADJ_STORE32
+  const unsigned tiles = blocks(a->lay.N), nt = 256;
+#else
+  const dim3 tiles((a->p.nx + AX - 1) / AX, (a->p.ny + AY - 1) / AY);
+  const unsigned nt = AX * AY;
+#endif
+  fwd_friction_kernel<<<blocks(a->lay.N), 256, 0, a->st>>>(a->p, Uin, Us, dt);
   store* rev = dptr(a, a->lay.off_rev);
   const long long r8 = 8 * (long long)a->lay.N;
-  fwd_stage_kernel<1><<<nb, 256, 0, a->st>>>(a->p, Us, nullptr, U1, m1, dt, t, hydro(a, t),
-                                             keep_rev ? rev : nullptr);
-  fwd_stage_kernel<2><<<nb, 256, 0, a->st>>>(a->p, Us, U1, Uout, m2, dt, t + dt, hydro(a, t + dt),
-                                             keep_rev ? rev + r8 : nullptr);
+  fwd_stage_kernel<1><<<tiles, nt, 0, a->st>>>(a->p, Us, nullptr, U1, m1, dt, t, hydro(a, t),
+                                                    keep_rev ? rev : nullptr);
+  fwd_stage_kernel<2><<<tiles, nt, 0, a->st>>>(a->p, Us, U1, Uout, m2, dt, t + dt,
+                                                    hydro(a, t + dt), keep_rev ? rev + r8 : nullptr);
   a->fwd_steps++;
   return launch_ok();
 }
 
 // Advances `buf` (the state after `from` steps) to the state after `to` steps.
 int advance(Ctx* a, store* buf, int from, int to) {
-  store* w = dptr(a, a->lay.off_work);
   double t = step_time(a, from);
-  const size_t s9 = (size_t)a->lay.plane9 * sizeof(store);
   for (int k = from; k < to; ++k) {
-    int r = fwd_step(a, k, t, buf, w);
+    int r = fwd_step(a, k, t, buf, buf);
     if (r) return r;
-    ACU(cudaMemcpyAsync(buf, w, s9, cudaMemcpyDeviceToDevice, a->st));
     t += a->dts[k];
   }
   return DG2_OK;
@@ -1755,7 +1965,6 @@ int forward_all(Ctx* a, double* loss) {
   ACU(cudaMemcpyAsync(cur, dptr(a, L.off_U0), s9, cudaMemcpyDeviceToDevice, a->st));
   const int ns = (int)a->samp_step.size();
   a->gauge_h.assign((size_t)ns * a->ngauge, 0.0);
-  store* w = dptr(a, L.off_work);
   double t = a->t0;
   auto sample = [&](int k) -> int {
     for (int s = 0; s < ns; ++s) {
@@ -1772,11 +1981,7 @@ int forward_all(Ctx* a, double* loss) {
   };
   int r = sample(0);
   for (int k = 0; k < K && !r; ++k) {
-    r = fwd_step(a, k, t, cur, w);
-    if (!r) {
-      cudaError_t e = cudaMemcpyAsync(cur, w, s9, cudaMemcpyDeviceToDevice, a->st);
-      if (e != cudaSuccess) r = afail(DG2_E_CUDA, "copy failed: %s", cudaGetErrorString(e));
-    }
+    r = fwd_step(a, k, t, cur, cur);
     t += a->dts[k];
     if (!r) r = sample(k + 1);
   }
@@ -1829,7 +2034,7 @@ int create(Ctx** out, int nx, int ny, double dx, double dy, const dg2_params* pr
   memset(&p, 0, sizeof p);
   p.nx = nx; p.ny = ny; p.N = L.N;
   p.dx = dx; p.dy = dy; p.inv_dx = 1.0 / dx; p.inv_dy = 1.0 / dy;
-  p.g = prm->g; p.tol = prm->tol_dry;
+  p.g = prm->g; p.tol = prm->tol_dry > 1e-300 ? prm->tol_dry : 1e-300;  // as a solver context
   p.wd = prm->wetdry == DG2_WD_POSITIVE ? 1 : 0;
   for (int k = 0; k < 4; ++k) p.bc[k] = prm->bc[k];
   p.in_edge = -1;

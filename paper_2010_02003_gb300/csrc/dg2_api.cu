@@ -560,9 +560,10 @@ int dg2_init_grid(dg2_ctx** out, int nx, int ny, double dx, double dy, const dg2
     const bool ll = p.variant == DG2_LL, f32 = p.precision == DG2_FP32;
     int o1 = 1, o2 = 1;
     // the FP64 stage tile's shared memory is above the 48 KB static limit
-    for (int k = 0; k < 8; ++k)
-      cudaFuncSetAttribute(stage64(k & 1, 1 + (k >> 1 & 1), k >> 2),
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(dg2::StageSmem));
+    if (!f32)
+      for (int stage = 1; stage <= 2; ++stage)
+        cudaFuncSetAttribute(stage64(ll, stage, p.flux == DG2_ROE),
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(dg2::StageSmem));
     if (f32) {
       dg2::ens::occupancy32(tile_w(c), ll, &o1, &o2);
     }

@@ -666,24 +666,23 @@ static __global__ void init_kernel(Dev d, const double* __restrict__ zc, const d
 // FP32 on the integer units) and the binomial series about it: h = (1 - e) / r^3 with
 // |e| < 1e-6, so h^(-7/3) = r^7 (1 + 7/3 e + 35/9 e^2 + O(6 e^3)), 8 FP64 instructions and
 // no conversion; two Newton steps on the root took about 20.  Outside, h^2 cbrt(h) divides.
+__device__ __forceinline__ double h_m73(double h) {
+  if (!(fbits(h) > fbits(1e-30) && fbits(h) < fbits(1e30))) return 1.0 / (h * h * cbrt(h));
+  const float hf = __int_as_float(((__double2hiint(h) - 0x38000000) << 3) |
+                                  (int)((unsigned)__double2loint(h) >> 29));
+  const int rb = __float_as_int(rcbrtf(hf));
+  const double r = __hiloint2double((rb >> 3) + 0x38000000, rb << 29);
+  const double r3 = r * r * r;
+  const double e = fma(-h, r3, 1.0);
+  const double r7 = r3 * r3 * r;
+  return fma(r7 * e, fma(35.0 / 9.0, e, 7.0 / 3.0), r7);
+}
 __device__ __forceinline__ void friction_point(double gn2dt, double tol, double h, double& qx,
                                                double& qy) {
   if (!above(h, tol)) return;
   const double qm = sqrt64(fma(qx, qx, qy * qy));
-  double iden;
-  if (fbits(h) > fbits(1e-30) && fbits(h) < fbits(1e30)) {
-    const float hf = __int_as_float(((__double2hiint(h) - 0x38000000) << 3) |
-                                    (int)((unsigned)__double2loint(h) >> 29));
-    const int rb = __float_as_int(rcbrtf(hf));
-    const double r = __hiloint2double((rb >> 3) + 0x38000000, rb << 29);
-    const double r3 = r * r * r;
-    const double e = fma(-h, r3, 1.0);
-    const double r7 = r3 * r3 * r;
-    const double hm73 = fma(r7 * e, fma(35.0 / 9.0, e, 7.0 / 3.0), r7);
-    iden = rcp64(fma(gn2dt * qm, hm73, 1.0));
-  } else {
-    iden = 1.0 / (1.0 + gn2dt * qm / (h * h * cbrt(h)));
-  }
+  const double den = fma(gn2dt * qm, h_m73(h), 1.0);
+  const double iden = above(den, 1e300) ? 0.0 : rcp64(den);
   qx = qx * iden;
   qy = qy * iden;
 }
@@ -806,6 +805,48 @@ struct StageK {
   double dx3, dy3;  // -3 dt / dx, -3 dt / dy
   double bx, by;    // -g dt / (2 dx), -g dt / (2 dy)
 };
+
+// Adds k L of Eqs. 4-5 to a cell's nine modes, with the step folded into the weights
+// (StageK), from its four faces (west, east, south, north) and its own side and pressure
+// step at the west and south ones (the lower sides of the others are with the faces).  The
+// own pressures and the bed terms of a direction share one product: with s, d the sum and
+// difference of the own face depths and r = d + zE - zW the step of the free surface
+// between the faces, Eq. 4a has -g s r / (2 dx) and Eqs. 4b-c (with the Gauss points'
+// pressures) -g d r / (2 dx) beside the pressure-free fluxes.  Small terms are summed
+// before they meet the base.
+__device__ __forceinline__ void apply_operator(const StageK& K, const FaceR& FW, const FaceR& FE,
+                                               const Side& W, double dpW, const FaceR& FS,
+                                               const FaceR& FN, const Side& S, double dpS,
+                                               double tol, double* out) {
+  const double tol2 = 2.0 * tol;
+  double l0, lx, ly;  // k L of the averages
+  {  // x direction
+    const Side E = FE.a;  // own side of the east face: its lower side
+    const double hs = E.h + W.h, hd = E.h - W.h;
+    const F3 G = gauss_pair(hs, E.qx + W.qx, E.qy + W.qy, hd, E.qx - W.qx, E.qy - W.qy, tol2);
+    const double bed = K.bx * (hd + (E.z - W.z));
+    const double eh = FE.h, wh = FW.h, en = FE.n, wn = FW.n + dpW, et = FE.t, wt = FW.t;
+    l0 = K.dx * (eh - wh);
+    lx = fma(K.dx, en - wn, bed * hs);
+    ly = K.dx * (et - wt);
+    out[H1X] = fma(K.dx3, fma(-0.5, G.h, eh + wh), out[H1X]);
+    out[QX1X] += fma(K.dx3, fma(-0.5, G.n, en + wn), bed * hd);
+    out[QY1X] = fma(K.dx3, fma(-0.5, G.t, et + wt), out[QY1X]);
+  }
+  {  // y direction
+    const Side N = FN.a;
+    const double hs = N.h + S.h, hd = N.h - S.h;
+    const F3 G = gauss_pair(hs, N.qy + S.qy, N.qx + S.qx, hd, N.qy - S.qy, N.qx - S.qx, tol2);
+    const double bed = K.by * (hd + (N.z - S.z));
+    const double nh = FN.h, sh = FS.h, nn = FN.n, sn = FS.n + dpS, nt = FN.t, st = FS.t;
+    out[H0] += fma(K.dy, nh - sh, l0);
+    out[QX0] += fma(K.dy, nt - st, lx);
+    out[QY0] += fma(bed, hs, fma(K.dy, nn - sn, ly));
+    out[H1Y] = fma(K.dy3, fma(-0.5, G.h, nh + sh), out[H1Y]);
+    out[QX1Y] = fma(K.dy3, fma(-0.5, G.t, nt + st), out[QX1Y]);
+    out[QY1Y] += fma(K.dy3, fma(-0.5, G.n, nn + sn), bed * hd);
+  }
+}
 
 struct StageSmem {
   Rec e[TY][TX];     // east record of each cell (lower side of the face to its east)
@@ -1201,14 +1242,8 @@ __device__ __forceinline__ void stage_tile(const Dev& d, StageSmem& sm, int bx, 
   __syncthreads();
   bool nq_out = false;  // the cell's output is non-quiescent
   if (act && b_me) {
-    // The stage's update is base + k L, k = dt and base = U^n in stage 1, k = dt / 2 and
-    // base = (U^n + U^1) / 2 in stage 2, with L of Eqs. 4-5 and the step folded into its
-    // weights (StageK).  The own pressures and the bed terms of a direction share one
-    // product: with s, d the sum and difference of the own face depths and r = d + zE - zW
-    // the step of the free surface between the faces, Eq. 4a has -g s r / (2 dx) and
-    // Eqs. 4b-c (with the Gauss points' pressures) -g d r / (2 dx) beside the
-    // pressure-free fluxes.  Small terms are summed before they meet the base.
-    const StageK K = sm.k;
+    // base + k L: k = dt and base = U^n in stage 1, k = dt / 2 and base = (U^n + U^1) / 2 in
+    // stage 2
     double out[9];
     if (STAGE == 1) {
 #pragma unroll
@@ -1227,38 +1262,8 @@ __device__ __forceinline__ void stage_tile(const Dev& d, StageSmem& sm, int bx, 
 #pragma unroll
       for (int k = 0; k < 9; ++k) out[k] = half64(out[k] + m[k]);
     }
-    const double tol2 = 2.0 * tol;
-    double l0, lx, ly;  // k L of the averages
-    {  // x direction
-      const FaceR& FW = sm.fx[ty][tx];
-      const FaceR& FE = sm.fx[ty][tx + 1];
-      const Side E = FE.a;  // own side of the east face: its lower side
-      const double hs = E.h + W.h, hd = E.h - W.h;
-      const F3 G = gauss_pair(hs, E.qx + W.qx, E.qy + W.qy, hd, E.qx - W.qx, E.qy - W.qy, tol2);
-      const double bed = K.bx * (hd + (E.z - W.z));
-      const double eh = FE.h, wh = FW.h, en = FE.n, wn = FW.n + dpW, et = FE.t, wt = FW.t;
-      l0 = K.dx * (eh - wh);
-      lx = fma(K.dx, en - wn, bed * hs);
-      ly = K.dx * (et - wt);
-      out[H1X] = fma(K.dx3, fma(-0.5, G.h, eh + wh), out[H1X]);
-      out[QX1X] += fma(K.dx3, fma(-0.5, G.n, en + wn), bed * hd);
-      out[QY1X] = fma(K.dx3, fma(-0.5, G.t, et + wt), out[QY1X]);
-    }
-    {  // y direction
-      const FaceR& FS = sm.fy[ty][tx];
-      const FaceR& FN = sm.fy[ty + 1][tx];
-      const Side N = FN.a;
-      const double hs = N.h + S.h, hd = N.h - S.h;
-      const F3 G = gauss_pair(hs, N.qy + S.qy, N.qx + S.qx, hd, N.qy - S.qy, N.qx - S.qx, tol2);
-      const double bed = K.by * (hd + (N.z - S.z));
-      const double nh = FN.h, sh = FS.h, nn = FN.n, sn = FS.n + dpS, nt = FN.t, st = FS.t;
-      out[H0] += fma(K.dy, nh - sh, l0);
-      out[QX0] += fma(K.dy, nt - st, lx);
-      out[QY0] += fma(bed, hs, fma(K.dy, nn - sn, ly));
-      out[H1Y] = fma(K.dy3, fma(-0.5, G.h, nh + sh), out[H1Y]);
-      out[QX1Y] = fma(K.dy3, fma(-0.5, G.t, nt + st), out[QX1Y]);
-      out[QY1Y] += fma(K.dy3, fma(-0.5, G.n, nn + sn), bed * hd);
-    }
+    apply_operator(sm.k, sm.fx[ty][tx], sm.fx[ty][tx + 1], W, dpW, sm.fy[ty][tx], sm.fy[ty + 1][tx],
+                   S, dpS, tol, out);
     if (d.rain != 0.0 && ts >= d.rain_t0 && ts < d.rain_t1)
       out[H0] += (STAGE == 1 ? dt : 0.5 * dt) * d.rain;
     if (c == d.src_idx) out[H0] += (STAGE == 1 ? dt : 0.5 * dt) * (d.qp * d.inv_dx * d.inv_dy);
