@@ -51,6 +51,21 @@ constexpr int kChunkMin = 16, kChunkMax = 1024;
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
+// Blocks per 32 x 8 tile of an FP64 context's lists.  The FP64 pipe takes a warp
+// instruction per 64 cycles from each of an SM's four schedulers, so a tile's 256 cells keep
+// an SM busy for 10 to 20 us a stage: finer blocks spread a short list over more SMs and
+// even out a long one, at the price of more records and faces on their edges.  Measured (us a step,
+// 32 -> 16 -> 8 columns a block; DG2-NL basins): 96^2 88.8, 64.5, 65.0; 128^2 88.7, 66.0,
+// 66.0; 256^2 143.6, 143.9, 135.6; 384^2 259.9, 257.0, 266.7; 1024^2 1618, 1607, 1658;
+// floodplains 500 x 300 136, 124, 107; 1237 x 731 317, 299, 308; 2000 x 1000 (DG2-LL) 259,
+// 250, 265.  So 16 columns, and 8 on grids of up to two tiles per SM.
+constexpr int kFineTiles = 304;
+int parts64(int nx, int ny, int scheme) {
+  if (scheme != DG2_SCHEME_DG2) return 1;
+  const long long nt = (long long)((nx + 31) / 32) * ((ny + 7) / 8);
+  return nt <= kFineTiles ? 4 : 2;
+}
+
 struct Layout {
   int pitch, zpx;
   long long plane;
@@ -72,7 +87,8 @@ bool make_layout(int nx, int ny, const dg2_params& p, Layout& L) {
   const size_t pb = (size_t)L.plane * esz;
   // set_dem stages the FP64 corner arrays and Manning field in the stage buffer
   const size_t staging = sizeof(double) * (2 * (size_t)(nx + 1) * (ny + 1) + (size_t)nx * ny);
-  const int tw = f32 ? (dg2::ens::f32_small_tiles((long long)nx * ny) ? 16 : 32) : dg2::TX;
+  const int tw = f32 ? (dg2::ens::f32_small_tiles((long long)nx * ny) ? 16 : 32)
+                     : dg2::TW;
   const int th = dg2::TY;
   L.nblocks = ((nx + tw - 1) / tw) * ((ny + th - 1) / th);
   L.mblocks = ((nx + 31) / 32) * ((ny + 7) / 8);
@@ -90,7 +106,8 @@ bool make_layout(int nx, int ny, const dg2_params& p, Layout& L) {
   L.off_ZX = take(f32 ? (size_t)ny * L.zpx * sizeof(float) : 0);
   L.off_ZY = take(f32 ? (size_t)(ny + 1) * L.pitch * sizeof(float) : 0);
   L.off_N = take(pb);
-  L.off_bpart = take(2 * (size_t)L.nblocks * sizeof(double));
+  const int parts = f32 ? 1 : parts64(nx, ny, p.scheme);
+  L.off_bpart = take(2 * (size_t)L.nblocks * parts * sizeof(double));
   L.off_mpart = take((size_t)L.mblocks * sizeof(double));
   L.off_kt = take((size_t)dg2::kMaxInflow * kMaxKnots * sizeof(double));
   L.off_kq = take((size_t)dg2::kMaxInflow * kMaxKnots * sizeof(double));
@@ -101,13 +118,13 @@ bool make_layout(int nx, int ny, const dg2_params& p, Layout& L) {
   L.off_st = take((size_t)p.max_samples * sizeof(double));
   L.off_sh = take((size_t)p.max_samples * ng * sizeof(double));
   L.off_sc = take(sizeof(Scalars));
-  L.off_tflag = take((size_t)L.nblocks);
+  L.off_tflag = take((size_t)L.nblocks * parts);
   L.off_tact = take((size_t)L.nblocks);
   L.off_tforced = take((size_t)L.nblocks);
   L.off_tlist = take((size_t)dg2::kListClasses * L.nblocks * sizeof(int));
   L.off_tfront = take((size_t)L.nblocks * sizeof(int));
   // FP64: the warp-block masks of Un and U1 and stage 1's computed blocks
-  L.nbx = (nx + dg2::TX - 1) / dg2::TX * dg2::TBX;
+  L.nbx = (nx + 31) / 32 * (32 / dg2::WX);
   L.nby = (ny + dg2::TY - 1) / dg2::TY * dg2::TBY;
   L.off_qm = take(f32 ? 0 : 3 * (size_t)L.nbx * L.nby * sizeof(unsigned));
   // FP32: the problem's descriptor and step counters for the shared FP32 kernels
@@ -137,7 +154,7 @@ struct dg2_ctx {
   // refused until dg2_set_dem / dg2_set_state give a valid state again
   int poisoned;
   int64_t launches;
-  dim3 sgrid, sblock, pgrid, pblock;
+  dim3 sblock, pgrid, pblock;
   int g_fric, g_st1, g_st2;   // persistent grid sizes (blocks) of friction / stage 1 / stage 2
   dg2::ens::EnsDev e1;        // FP32: this problem as a set of one for the shared FP32 kernels
   dim3 lgrid, lblock;          // lists_kernel: one thread per tile
@@ -155,7 +172,7 @@ namespace {
 // Cells per tile of the context's dry-tile skipping: 32 x 8 for the FP64
 // kernels; 16 x 8 or 32 x 8 for a single FP32 problem by its size.
 int tile_w(const dg2_ctx* c) {
-  return c->fp32 && dg2::ens::f32_small_tiles((long long)c->d.nx * c->d.ny) ? 16 : dg2::TX;
+  return c->fp32 && dg2::ens::f32_small_tiles((long long)c->d.nx * c->d.ny) ? 16 : dg2::TW;
 }
 int tile_h(const dg2_ctx*) { return dg2::TY; }
 
@@ -252,19 +269,26 @@ void mirror(dg2_ctx* c) {
   f.tiles = d.tiles;
 }
 
-// The FP64 DG2 stage kernel of a variant, stage and Riemann solver.
+// The FP64 DG2 stage kernel of a variant, stage, Riemann solver and width of a block.
 using StageFn = void (*)(Dev);
-StageFn stage64(bool ll, int stage, bool roe) {
+template <int TX>
+StageFn stage64_of(bool ll, int stage, bool roe) {
   if (roe) {
-    if (ll) return stage == 1 ? dg2::stage_kernel<true, 1, true> : dg2::stage_kernel<true, 2, true>;
-    return stage == 1 ? dg2::stage_kernel<false, 1, true> : dg2::stage_kernel<false, 2, true>;
+    if (ll) return stage == 1 ? dg2::stage_kernel<true, 1, true, TX> : dg2::stage_kernel<true, 2, true, TX>;
+    return stage == 1 ? dg2::stage_kernel<false, 1, true, TX> : dg2::stage_kernel<false, 2, true, TX>;
   }
-  if (ll) return stage == 1 ? dg2::stage_kernel<true, 1, false> : dg2::stage_kernel<true, 2, false>;
-  return stage == 1 ? dg2::stage_kernel<false, 1, false> : dg2::stage_kernel<false, 2, false>;
+  if (ll) return stage == 1 ? dg2::stage_kernel<true, 1, false, TX> : dg2::stage_kernel<true, 2, false, TX>;
+  return stage == 1 ? dg2::stage_kernel<false, 1, false, TX> : dg2::stage_kernel<false, 2, false, TX>;
 }
-void launch_stage64(dg2_ctx* c, bool ll, int stage) {
-  stage64(ll, stage, c->d.flux == DG2_ROE)<<<stage == 1 ? c->g_st1 : c->g_st2, c->sblock,
-                                             sizeof(dg2::StageSmem), c->st>>>(c->d);
+StageFn stage64(const dg2_ctx* c, int stage) {
+  const bool ll = c->p.variant == DG2_LL, roe = c->d.flux == DG2_ROE;
+  return c->d.nsub == 4 ? stage64_of<8>(ll, stage, roe) : stage64_of<16>(ll, stage, roe);
+}
+size_t stage64_smem(const dg2_ctx* c) {
+  return c->d.nsub == 4 ? sizeof(dg2::StageSmem<8>) : sizeof(dg2::StageSmem<16>);
+}
+void launch_stage64(dg2_ctx* c, int stage) {
+  stage64(c, stage)<<<stage == 1 ? c->g_st1 : c->g_st2, c->sblock, stage64_smem(c), c->st>>>(c->d);
 }
 
 // Enqueues one RK2 step: friction, stage 1, stage 2, finalize, lists (5 kernels; 4 in
@@ -285,7 +309,11 @@ void enqueue_step(dg2_ctx* c, bool timed = false) {
   const bool ll = c->p.variant == DG2_LL;
   if (e) cudaEventRecord(e[0], c->st);
   // FP32: friction is fused into the stage kernels (no launch of its own)
-  if (!c->fp32) dg2::friction_kernel<<<c->g_fric, c->sblock, 0, c->st>>>(d);
+  if (!c->fp32) {
+    if (d.nsub == 4) dg2::friction_kernel<8><<<c->g_fric, c->sblock, 0, c->st>>>(d);
+    else if (d.nsub == 2) dg2::friction_kernel<16><<<c->g_fric, c->sblock, 0, c->st>>>(d);
+    else dg2::friction_kernel<32><<<c->g_fric, c->sblock, 0, c->st>>>(d);
+  }
   if (e) cudaEventRecord(e[1], c->st);
   if (c->p.scheme != DG2_SCHEME_DG2) {
     // the FV comparators: one block per tile of the lists, as the DG2 stages
@@ -305,13 +333,13 @@ void enqueue_step(dg2_ctx* c, bool timed = false) {
   if (c->fp32) {
     dg2::ens::launch_stage32(c->e1, tile_w(c), ll, 1, c->g_st1, c->st);
   } else {
-    launch_stage64(c, ll, 1);
+    launch_stage64(c, 1);
   }
   if (e) cudaEventRecord(e[2], c->st);
   if (c->fp32) {
     dg2::ens::launch_stage32(c->e1, tile_w(c), ll, 2, c->g_st2, c->st);
   } else {
-    launch_stage64(c, ll, 2);
+    launch_stage64(c, 2);
   }
   if (e) cudaEventRecord(e[3], c->st);
   launch_finalize(c, 0);
@@ -353,7 +381,7 @@ void launch_mass(dg2_ctx* c) {
 // Marks every tile non-quiescent so the next step computes the whole grid
 // (after a new DEM or state; the first stage 2 then sets the true flags).
 int reset_tiles(dg2_ctx* c) {
-  CU(cudaMemsetAsync(c->d.tiles.flag, 1, (size_t)c->lay.nblocks, c->st));
+  CU(cudaMemsetAsync(c->d.tiles.flag, 1, (size_t)c->lay.nblocks * c->d.nsub, c->st));
   // every cell non-quiescent in the cell masks: the first step computes every cell
   if (c->d.qm)
     CU(cudaMemsetAsync(c->d.qm, 0xff, 3 * (size_t)c->d.qplane * sizeof(unsigned), c->st));
@@ -509,6 +537,7 @@ int dg2_init_grid(dg2_ctx** out, int nx, int ny, double dx, double dy, const dg2
   d.max_samples = p.max_samples;
   d.src_idx = -1;
   d.nblocks = L.nblocks;
+  d.nsub = c->fp32 ? 1 : parts64(nx, ny, p.scheme);
   d.tiles.flag = (unsigned char*)(c->ws + L.off_tflag);
   d.tiles.act = (unsigned char*)(c->ws + L.off_tact);
   d.tiles.forced = (const unsigned char*)(c->ws + L.off_tforced);
@@ -548,8 +577,7 @@ int dg2_init_grid(dg2_ctx** out, int nx, int ny, double dx, double dy, const dg2
     f.tiles = d.tiles;
     f.wd = d.wd;
   }
-  c->sblock = dim3(dg2::TX, dg2::TY);
-  c->sgrid = dim3((nx + dg2::TX - 1) / dg2::TX, (ny + dg2::TY - 1) / dg2::TY);
+  c->sblock = dim3(dg2::TW / d.nsub, dg2::TY);
   c->pblock = dim3(32, 8);
   c->pgrid = dim3((nx + 31) / 32, (ny + 7) / 8);
   {
@@ -561,9 +589,9 @@ int dg2_init_grid(dg2_ctx** out, int nx, int ny, double dx, double dy, const dg2
     int o1 = 1, o2 = 1;
     // the FP64 stage tile's shared memory is above the 48 KB static limit
     if (!f32)
-      for (int stage = 1; stage <= 2; ++stage)
-        cudaFuncSetAttribute(stage64(ll, stage, p.flux == DG2_ROE),
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(dg2::StageSmem));
+      for (int stage = 1; stage <= 2 && p.scheme == DG2_SCHEME_DG2; ++stage)
+        cudaFuncSetAttribute(stage64(c, stage), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)stage64_smem(c));
     if (f32) {
       dg2::ens::occupancy32(tile_w(c), ll, &o1, &o2);
     }
@@ -575,9 +603,9 @@ int dg2_init_grid(dg2_ctx** out, int nx, int ny, double dx, double dy, const dg2
     // friction: one block per tile of the list (the hardware hands blocks to SMs
     // as they free up); measured faster than a persistent grid looping over the
     // list (floodplain 2000 x 1000 from t = 1 h: 0.060 -> 0.051 ms per step)
-    c->g_fric = nt;
-    c->g_st1 = f32 ? gsz(o1) : nt;
-    c->g_st2 = f32 ? gsz(o2) : nt;
+    c->g_fric = nt * d.nsub;
+    c->g_st1 = f32 ? gsz(o1) : nt * d.nsub;
+    c->g_st2 = f32 ? gsz(o2) : nt * d.nsub;
   }
 
   // zero the state, topography and scalars; t_end / samples at +inf

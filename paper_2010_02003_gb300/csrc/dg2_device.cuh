@@ -22,23 +22,19 @@
 
 namespace dg2 {
 
-// FP64 tile of TX x TY cells.  Measured on GB300 with the weight-class lists
-// (floodplain 2000 x 1000 from t = 1 h, ms per step, 32 -> 16 wide): DG2-LL
-// 0.421 -> 0.422, DG2-NL 0.345 -> 0.335; 32 x 8 is kept.
-#ifndef DG2_TX64
-#define DG2_TX64 32
-#endif
-constexpr int TX = DG2_TX64;
+// The tiles of the FP64 lists are TW x TY = 32 x 8 cells.  A block of the DG2 kernels works
+// on a part of one, TX x TY cells (TX a template parameter, TW / TX parts a tile,
+// Dev::nsub; the FV kernels take whole tiles).  A warp covers a WX x WY block of cells
+// (lane l: column l % WX, row l / WX of the block); a part is TX / 8 x 2 such blocks, warp w
+// the block (w % (TX / 8), w / (TX / 8)).  Wet regions are compact, so square-ish blocks
+// hold fewer dry lanes than rows of 32.  The cell of the calling thread in its part:
+constexpr int TW = 32;
 constexpr int TY = 8;
-
-// A warp of the FP64 tile kernels covers a WX x WY block of cells (lane l:
-// column l % WX, row l / WX of the block); a 32 x 8 tile is 4 x 2 such blocks,
-// warp w the block (w % 4, w / 4).  Wet regions are compact, so square-ish
-// blocks hold fewer dry lanes than rows of 32.  The tile cell of the calling
-// thread:
-constexpr int WX = 8, WY = 4, TBX = TX / WX, TBY = TY / WY;
-static_assert(WX * WY == 32 && TBX * WX == TX && TBY * WY == TY, "warp blocks tile the tile");
+constexpr int WX = 8, WY = 4, TBY = TY / WY;
+template <int TX>
 __device__ __forceinline__ void warp_cell(int& tx, int& ty) {
+  constexpr int TBX = TX / WX;
+  static_assert(WX * WY == 32 && TBX * WX == TX && TBY * WY == TY, "warp blocks tile the tile");
   const int t = threadIdx.y * TX + threadIdx.x, w = t >> 5, l = t & 31;
   tx = (w % TBX) * WX + (l % WX);
   ty = (w / TBX) * WY + (l / WX);
@@ -123,7 +119,8 @@ struct Scalars {
 // friction skips 8 x 4 warp blocks of quiescent cells.  Forced tiles, rain and
 // skip = 0 compute every cell.
 struct Tiles {
-  unsigned char* flag;          // [ntiles] tile held a non-quiescent cell after the last stage 2
+  unsigned char* flag;          // [ntiles * parts] part of a tile held a non-quiescent cell
+                                // after the last stage 2 (parts: 1, FP64 DG2 Dev::nsub)
   unsigned char* act;           // [ntiles] tile computed in the current step
   const unsigned char* forced;  // [ntiles] tile must be computed (inflow, source); set on the host
   int* list;                    // [kListClasses * ntiles] computed tiles of the step, by weight class
@@ -171,7 +168,7 @@ struct Dev {
   double* Q;                 // 6 planes: limited slopes of Un (DG2-LL)
   const double* Z;           // 3 planes: z0, z1x, z1y
   const double* N;           // 1 plane: Manning n
-  double* bpart;             // [2][nblocks] boundary mass-rate partials
+  double* bpart;             // [2][ntiles * nsub] boundary mass-rate partials
   double* mpart;             // [nblocks] mass partials
   Scalars* sc;
   // gauges
@@ -188,9 +185,12 @@ struct Dev {
   // (plane 0, written by stage 2) and of U1 (plane 1, by stage 1), and the
   // cells stage 1 computed (plane 2)
   unsigned int* qm;
-  int nbx, nby;              // warp blocks per row / column (whole tiles)
+  int nbx, nby;              // warp blocks per row / column (whole 32 x 8 tiles)
+  int nsub;                  // blocks (parts) per tile: 1, FP64 DG2 2 or 4 (parts64)
   long long qplane;          // words per qm plane
 };
+
+__device__ __forceinline__ int parts_of(const Dev& d) { return d.nsub; }
 
 // ---------------------------------------------------------------------------
 // FP64 comparisons on the integer units
@@ -687,17 +687,19 @@ __device__ __forceinline__ void friction_point(double gn2dt, double tol, double 
   qy = qy * iden;
 }
 
-// Friction on the cells of one 32 x 8 tile (threads 32 x 8).  A quiescent cell
+// Friction on the cells of one tile (one thread each).  A quiescent cell
 // (every Gauss-point depth at h0 <= tol_dry, Un's qm bit clear) has no water to
 // rub, and neither has a cell without roughness: the others are gathered and
 // handed to the first threads, so the FP64 arithmetic runs on full warps.
 // `cells` is shared memory for the tile's list, `cnt` for the per-warp counts.
+template <int TX>
 __device__ __forceinline__ void friction_tile(const Dev& d, int bx, int by, unsigned short* cells,
                                               int* cnt) {
   const Scalars* sc = d.sc;
   const int t = threadIdx.y * TX + threadIdx.x, w = t >> 5, lane = t & 31;
+  constexpr int TBX = TX / WX;
   int tx, ty;
-  warp_cell(tx, ty);
+  warp_cell<TX>(tx, ty);
   const int i = bx * TX + tx, j = by * TY + ty;
   const long long P = d.plane;
   bool work = i < d.nx && j < d.ny;
@@ -753,10 +755,11 @@ __device__ __forceinline__ void friction_tile(const Dev& d, int bx, int by, unsi
     S[QX1Y * P + c] = nq[1][0];
     S[QY1Y * P + c] = nq[1][1];
   }
-  __syncthreads();  // the list is reused by the block's next tile
 }
 
-// Friction over the step's computed tiles (a quiescent tile has no water to rub).
+// Friction over the step's computed tiles (a quiescent tile has no water to rub), one block
+// per part of a tile.
+template <int TX>
 static __global__ void __launch_bounds__(TX * TY) friction_kernel(Dev d) {
   __shared__ unsigned short cells[TX * TY];
   __shared__ int cnt[TX * TY / 32];
@@ -764,10 +767,11 @@ static __global__ void __launch_bounds__(TX * TY) friction_kernel(Dev d) {
   if (sc->done) return;
   const int n_act = sc->n_act, ntx = d.tiles.ntx;
   const bool all = sc->list_all != 0;
-  for (int e = blockIdx.x; e < n_act; e += gridDim.x) {
-    const int tile = all ? e : list_tile(d.tiles, sc, e);
-    friction_tile(d, tile % ntx, tile / ntx, cells, cnt);
-  }
+  constexpr int PARTS = TW / TX;
+  const int e = blockIdx.x / PARTS;
+  if (e >= n_act) return;
+  const int tile = all ? e : list_tile(d.tiles, sc, e);
+  friction_tile<TX>(d, tile % ntx * PARTS + blockIdx.x % PARTS, tile / ntx, cells, cnt);
 }
 
 // Loads the 9 coefficients of cell c from buffer U.
@@ -848,6 +852,7 @@ __device__ __forceinline__ void apply_operator(const StageK& K, const FaceR& FW,
   }
 }
 
+template <int TX>
 struct StageSmem {
   Rec e[TY][TX];     // east record of each cell (lower side of the face to its east)
   Rec n[TY][TX];     // north record of each cell
@@ -1032,14 +1037,15 @@ __device__ __forceinline__ Rec ghost_rec(const Dev& d, int edge, double s, doubl
 // which also build the halo records.  Forced tiles, rain and skip = 0 compute
 // every cell.  Returns the calling thread's cell in (tx, ty); sm.cls[y][x]
 // holds each cell's class (0 outside the grid, 1 fixed point, 2 computed).
-template <int STAGE>
-__device__ __forceinline__ void classify_cells(const Dev& d, StageSmem& sm, int bx, int by,
+template <int STAGE, int TX>
+__device__ __forceinline__ void classify_cells(const Dev& d, StageSmem<TX>& sm, int bx, int by,
                                                bool every, int& tx, int& ty) {
+  constexpr int TBX = TX / WX;
   const int t = threadIdx.y * TX + threadIdx.x, w = t >> 5, lane = t & 31;
   // the input's non-quiescence of the tile's cells and of the ring around it
   {
     int cx, cy;
-    warp_cell(cx, cy);
+    warp_cell<TX>(cx, cy);
     const int X = bx * TBX + cx / WX, Y = by * TBY + cy / WY;
     const unsigned* qm = STAGE == 1 ? d.qm : d.qm + d.qplane;
     const bool in = bx * TX + cx < d.nx && by * TY + cy < d.ny;
@@ -1061,7 +1067,7 @@ __device__ __forceinline__ void classify_cells(const Dev& d, StageSmem& sm, int 
   }
   __syncthreads();
   int cx, cy;
-  warp_cell(cx, cy);
+  warp_cell<TX>(cx, cy);
   const bool act = bx * TX + cx < d.nx && by * TY + cy < d.ny;
   bool comp = false;
   if (act) {
@@ -1106,17 +1112,17 @@ __device__ __forceinline__ void classify_cells(const Dev& d, StageSmem& sm, int 
   ty = me / TX;
 }
 
-// One RK stage on the 32 x 8 tile (bx, by): face records, one revision and
+// One RK stage on the TX x 8 part (bx, by) of tile `tile`: face records, one revision and
 // one flux per face, Eqs. 4-5, the stage update and the wet-dry treatment.
 // Accumulates the boundary inflow rate, the Courant rate and the non-finite /
 // non-quiescent flags of the thread's cell into the caller's variables.  Cells
 // that are fixed points of the stage (classify_cells) skip the faces and
 // Eqs. 4-5.
-template <bool LL, int STAGE, bool ROE>
-__device__ __forceinline__ void stage_tile(const Dev& d, StageSmem& sm, int bx, int by,
-                                           double& brate, double& lam, bool& bad, bool& nonq) {
+template <bool LL, int STAGE, bool ROE, int TX>
+__device__ __forceinline__ void stage_tile(const Dev& d, StageSmem<TX>& sm, int bx, int by,
+                                           int tile, double& brate, double& lam, bool& bad, bool& nonq) {
+  constexpr int TBX = TX / WX;
   Scalars* sc = d.sc;
-  const int tile = by * d.tiles.ntx + bx;
   const bool every = !d.tiles.skip || d.tiles.all_forced || d.tiles.forced[tile];
   const double dt = sc->dt;
   if (threadIdx.x == 0 && threadIdx.y == 0) {
@@ -1125,7 +1131,7 @@ __device__ __forceinline__ void stage_tile(const Dev& d, StageSmem& sm, int bx, 
                   -0.5 * d.g * k * d.inv_dx, -0.5 * d.g * k * d.inv_dy};
   }
   int tx, ty;
-  classify_cells<STAGE>(d, sm, bx, by, every, tx, ty);
+  classify_cells<STAGE, TX>(d, sm, bx, by, every, tx, ty);
   const int i = bx * TX + tx, j = by * TY + ty;
   const bool act = i < d.nx && j < d.ny;
   const long long P = d.plane;
@@ -1310,7 +1316,7 @@ __device__ __forceinline__ void stage_tile(const Dev& d, StageSmem& sm, int bx, 
   __syncthreads();
   {
     int cx, cy;
-    warp_cell(cx, cy);
+    warp_cell<TX>(cx, cy);
     const unsigned bits = __ballot_sync(0xffffffffu, sm.nqo[cy][cx] != 0);
     if ((threadIdx.x & 31) == 0) {
       const int X = bx * TBX + cx / WX, Y = by * TBY + cy / WY;
@@ -1333,23 +1339,17 @@ __device__ __forceinline__ void stage_tile(const Dev& d, StageSmem& sm, int bx, 
 // 44.8 ms, the 128 x 128 basin 13.5 -> 10.9 ms, with errors against an 80-bit run of the
 // same scheme 1.0 to 0.9 of what they were.
 //
-// minimum resident blocks per SM asked of the register allocator: 2 for both
-// FP64 stages (128 registers; measured on the floodplain, DG2-LL 0.857 ms/step
-// at 2 blocks against 0.955 at 1 block with 156 registers)
-#ifndef DG2_MINB64_NL
-#define DG2_MINB64_NL 2
-#endif
-#ifndef DG2_MINB64_LL
-#define DG2_MINB64_LL 2
-#endif
-
+// 16 resident warps per SM are asked of the register allocator (128 registers a thread;
+// 2 blocks of 32 x 8 cells measured faster than 1 with 156 registers: DG2-LL floodplain
+// 0.857 against 0.955 ms per step).
 // Stage kernels run over the step's list of active tiles (and, in stage 1,
 // the frontier tiles that only copy their state for a neighbour's halo),
 // built at the end of the previous step.
-template <bool LL, int STAGE, bool ROE>
-static __global__ void __launch_bounds__(TX* TY, LL ? DG2_MINB64_LL : DG2_MINB64_NL) stage_kernel(Dev d) {
-  extern __shared__ double stage_smem[];  // one StageSmem (dynamic: above 48 KB)
-  StageSmem& sm = *reinterpret_cast<StageSmem*>(stage_smem);
+template <bool LL, int STAGE, bool ROE, int TX>
+static __global__ void __launch_bounds__(TX* TY, 2 * TW / TX) stage_kernel(Dev d) {
+  constexpr int TBX = TX / WX, PARTS = TW / TX;
+  extern __shared__ double stage_smem[];  // one StageSmem (dynamic: may pass 48 KB)
+  StageSmem<TX>& sm = *reinterpret_cast<StageSmem<TX>*>(stage_smem);
   Scalars* sc = d.sc;
   if (sc->done) return;
   const int tx = threadIdx.x, ty = threadIdx.y;
@@ -1358,23 +1358,31 @@ static __global__ void __launch_bounds__(TX* TY, LL ? DG2_MINB64_LL : DG2_MINB64
   const bool all = sc->list_all != 0;
   double lam = 0.0;
   bool bad = false;
-  if (STAGE == 2 && (int)blockIdx.x >= n_act) return;
-  if ((int)blockIdx.x < n_act) {
-    const int e = blockIdx.x;
+  const int e = blockIdx.x / PARTS, part = blockIdx.x % PARTS;
+  if (STAGE == 2 && e >= n_act) return;
+  if (e < n_act) {
     const int tile = all ? e : list_tile(d.tiles, sc, e);
-    const int bx = tile % ntx, by = tile / ntx;
-    double brate = 0.0, lam_t = 0.0;
+    const int tbx = tile % ntx, by = tile / ntx;
+    double brate = 0.0;
     bool nonq = false;
-    stage_tile<LL, STAGE, ROE>(d, sm, bx, by, brate, lam_t, bad, nonq);
-    lam = fmax(lam, lam_t);
-    // boundary inflow rate of an edge tile, kept per tile (summed in tile order later)
-    if (bx == 0 || by == 0 || bx == ntx - 1 || by == d.tiles.nty - 1) {
+    const int bx = tbx * PARTS + part;
+    if (bx * TX < d.nx) {
+      stage_tile<LL, STAGE, ROE, TX>(d, sm, bx, by, tile, brate, lam, bad, nonq);
+    } else if ((threadIdx.y * TX + threadIdx.x) % 32 == 0) {
+      // a part wholly past the grid's east edge: no cells, clear mask bits
+      int cx, cy;
+      warp_cell<TX>(cx, cy);
+      d.qm[(STAGE == 1 ? d.qplane : 0) + (long long)(by * TBY + cy / WY) * d.nbx + bx * TBX +
+           cx / WX] = 0u;
+    }
+    // boundary inflow rate of an edge tile, kept per part (summed in tile order later)
+    if (tbx == 0 || by == 0 || tbx == ntx - 1 || by == d.tiles.nty - 1) {
       const double bsum = block_sum<TX * TY>(brate, sm.red);
-      if (tx == 0 && ty == 0) d.bpart[(STAGE - 1) * d.tiles.ntiles + tile] = bsum;
+      if (tx == 0 && ty == 0) d.bpart[((STAGE - 1) * d.tiles.ntiles + tile) * PARTS + part] = bsum;
     }
     if (STAGE == 2) {
       const int any_nonq = __syncthreads_or(nonq);
-      if (tx == 0 && ty == 0) d.tiles.flag[tile] = any_nonq ? 1 : 0;
+      if (tx == 0 && ty == 0) d.tiles.flag[tile * PARTS + part] = any_nonq ? 1 : 0;
     }
     __syncthreads();
   }
@@ -1382,12 +1390,13 @@ static __global__ void __launch_bounds__(TX* TY, LL ? DG2_MINB64_LL : DG2_MINB64
     // frontier tiles: a computed neighbour reads their stage state as halo
     const int n_front = sc->n_front;
     const long long P = d.plane;
-    const int e = (int)blockIdx.x - n_act;
-    if (e >= 0 && e < n_front) {
-      const int tile = d.tiles.front[e];
+    const int f = e - n_act;
+    if (f >= 0 && f < n_front) {
+      const int tile = d.tiles.front[f];
+      const int bx = tile % ntx * PARTS + part, by = tile / ntx;
       int cx, cy;
-      warp_cell(cx, cy);
-      const int i = (tile % ntx) * TX + cx, j = (tile / ntx) * TY + cy;
+      warp_cell<TX>(cx, cy);
+      const int i = bx * TX + cx, j = by * TY + cy;
       bool nq = false;
       if (i < d.nx && j < d.ny) {
         const long long c = (long long)j * d.pitch + i;
@@ -1401,7 +1410,7 @@ static __global__ void __launch_bounds__(TX* TY, LL ? DG2_MINB64_LL : DG2_MINB64
       // U1's non-quiescence bits of the copied blocks, for a computed neighbour's stage 2
       const unsigned bits = __ballot_sync(0xffffffffu, nq);
       if ((threadIdx.x & 31) == 0) {
-        const int X = (tile % ntx) * TBX + cx / WX, Y = (tile / ntx) * TBY + cy / WY;
+        const int X = bx * TBX + cx / WX, Y = by * TBY + cy / WY;
         d.qm[d.qplane + (long long)Y * d.nbx + X] = bits;
       }
     }
@@ -1428,8 +1437,7 @@ constexpr int kFinThreads = 1024;
 // bpart slot and flag, and the step's reductions are exact (max) or summed
 // per tile in a fixed order, so the step's result does not depend on it.
 constexpr int LTX = 32, LTY = 8;
-template <class D>
-static __global__ void __launch_bounds__(LTX* LTY) lists_kernel(D d) {
+static __global__ void __launch_bounds__(LTX* LTY) lists_kernel(Dev d) {
   Scalars* sc = d.sc;
   if (sc->skip_lists) return;
   const Tiles& T = d.tiles;
@@ -1455,7 +1463,8 @@ static __global__ void __launch_bounds__(LTX* LTY) lists_kernel(D d) {
     unsigned char v = 0;
     if (gx >= 0 && gy >= 0 && gx < ntx && gy < nty) {
       const int q = gy * ntx + gx;
-      v = (T.flag[q] | T.forced[q]) != 0;
+      v = T.forced[q];
+      for (int k = 0; k < d.nsub; ++k) v |= T.flag[q * d.nsub + k];
     }
     busy[ly][lx] = v;
   }
@@ -1480,9 +1489,9 @@ static __global__ void __launch_bounds__(LTX* LTY) lists_kernel(D d) {
   if (a && d.qm && d.scheme == 0) {
     int nq = 0;
     for (int yy = 0; yy < TBY; ++yy)
-      for (int xx = 0; xx < TBX; ++xx)
-        nq += __popc(d.qm[(long long)(by * TBY + yy) * d.nbx + bx * TBX + xx]);
-    cls = kListClasses - 1 - nq * kListClasses / (TX * TY + 1);
+      for (int xx = 0; xx < TW / WX; ++xx)
+        nq += __popc(d.qm[(long long)(by * TBY + yy) * d.nbx + bx * (TW / WX) + xx]);
+    cls = kListClasses - 1 - nq * kListClasses / (TW * TY + 1);
   }
   // warp = one row of LTX tiles: ballot prefix in the warp, warp offsets, one
   // atomic per class
@@ -1549,7 +1558,9 @@ static __device__ double ring_inflow(const D& d) {
     else if (k < 2 * ntx) t = (nty - 1) * ntx + (k - ntx);         // north row
     else if (k < 2 * ntx + nty - 2) t = (k - 2 * ntx + 1) * ntx;   // west column
     else t = (k - 2 * ntx - nty + 3) * ntx + ntx - 1;              // east column
-    if (T.act[t]) part += d.bpart[t] + d.bpart[nt + t];
+    if (T.act[t])
+      for (int k = 0, n = parts_of(d); k < n; ++k)
+        part += d.bpart[t * n + k] + d.bpart[(nt + t) * n + k];
   }
   return block_sum<kFinThreads>(part, red);
 }

@@ -72,6 +72,8 @@ struct __align__(16) D32 {
   int wd;              // 1: positivity-consistent revision of partially wet cells
 };
 
+__device__ __forceinline__ int parts_of(const D32&) { return 1; }
+
 struct LimF {
   float h, qx, qy, u, v;
 };

@@ -29,6 +29,7 @@
 namespace dg2 {
 namespace fv {
 
+constexpr int TX = TW;                   // a block takes a whole tile
 constexpr int HX = TX + 4, HY = TY + 4;  // staged region: tile + 2-cell halo
 
 struct L4 {
@@ -157,7 +158,7 @@ __device__ __forceinline__ void fv_tile(const Dev& d, Smem& sm, int bx, int by, 
   const Scalars* sc = d.sc;
   const int tid = threadIdx.y * TX + threadIdx.x;
   int tx, ty;
-  warp_cell(tx, ty);
+  warp_cell<TX>(tx, ty);
   const int i0 = bx * TX, j0 = by * TY, i = i0 + tx, j = j0 + ty;
   const int nx = d.nx, ny = d.ny;
   const bool act = i < nx && j < ny;
