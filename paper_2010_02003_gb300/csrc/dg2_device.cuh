@@ -566,24 +566,6 @@ __device__ __forceinline__ double block_max(double v, double* sh) {
   return r;
 }
 
-template <int NT>
-__device__ __forceinline__ float block_max_f(float v, float* sh) {
-  const int lane = (threadIdx.y * blockDim.x + threadIdx.x) & 31;
-  const int warp = (threadIdx.y * blockDim.x + threadIdx.x) >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_down_sync(0xffffffffu, v, o));
-  __syncthreads();
-  if (lane == 0) sh[warp] = v;
-  __syncthreads();
-  float r = 0.f;
-  if (warp == 0) {
-    r = lane < NT / 32 ? sh[lane] : 0.f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) r = fmaxf(r, __shfl_down_sync(0xffffffffu, r, o));
-  }
-  return r;
-}
-
 // Courant wave-speed rate of a cell: max((|u|+c)/dx, (|v|+c)/dy) if wet.
 __device__ __forceinline__ double cell_rate(const Dev& d, double h0, double qx0, double qy0) {
   if (!above(h0, d.tol)) return 0.0;

@@ -94,7 +94,6 @@ struct __align__(16) StagedSmem32 {
   RecF n[BY][BX];
   RecF hw[BY], he[BY], hs[BX], hn[BX];
   double red[32];
-  float redf[32];
 };
 
 // Friction of one cell's modes (Sec. 2.1.3): the point-implicit update at the
