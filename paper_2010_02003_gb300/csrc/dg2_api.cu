@@ -201,12 +201,18 @@ int sync_desc(dg2_ctx* c) {
   return DG2_OK;
 }
 
+// Kernels of the end of step (and of lists_only).
+int finalize_kernels(const dg2_ctx* c) {
+  return !c->fp32 && c->d.tiles.ntiles <= dg2::kSmallTiles ? 1 : 2;
+}
 // End of step (time, ledger, gauges, next dt) and the next step's tile lists
-// (2 kernels); with lists_only, just the lists (after a new DEM / state /
+// (finalize_kernels launches); with lists_only, just the lists (after a new DEM / state /
 // forced mask).
 void launch_finalize(dg2_ctx* c, int lists_only) {
   if (c->fp32) {
     dg2::ens::launch_end_of_step(c->e1, 1, c->lgrid, lists_only, c->st);
+  } else if (finalize_kernels(c) == 1) {
+    dg2::finalize_small_kernel<<<1, dg2::kFinThreads, 0, c->st>>>(c->d, lists_only);
   } else {
     dg2::finalize_kernel<<<1, dg2::kFinThreads, 0, c->st>>>(c->d, lists_only);
     dg2::lists_kernel<<<c->lgrid, c->lblock, 0, c->st>>>(c->d);
@@ -249,7 +255,7 @@ int update_forced_tiles(dg2_ctx* c) {
   CU(cudaMemcpyAsync((void*)d.tiles.forced, m.data(), m.size(), cudaMemcpyHostToDevice, c->st));
   if (c->dem_set) {
     launch_finalize(c, 1);   // the computed set depends on the forced mask
-    int r = launch_check(c, 2);
+    int r = launch_check(c, finalize_kernels(c));
     if (r) return r;
   }
   CU(cudaStreamSynchronize(c->st));
@@ -291,9 +297,11 @@ void launch_stage64(dg2_ctx* c, int stage) {
   stage64(c, stage)<<<stage == 1 ? c->g_st1 : c->g_st2, c->sblock, stage64_smem(c), c->st>>>(c->d);
 }
 
-// Enqueues one RK2 step: friction, stage 1, stage 2, finalize, lists (5 kernels; 4 in
-// FP32, whose stages apply friction themselves).  With `timed`, records an event before
-// and after each kernel.
+// Kernels of one RK2 step: friction (FP64; the FP32 stages apply it themselves), two stages,
+// the end of step.
+int step_kernels(const dg2_ctx* c) { return (c->fp32 ? 2 : 3) + finalize_kernels(c); }
+// Enqueues one RK2 step.  With `timed`, records an event before and after each of friction
+// and the stages.
 void enqueue_step(dg2_ctx* c, bool timed = false) {
   const Dev& d = c->d;
   cudaEvent_t* e = nullptr;
@@ -386,7 +394,7 @@ int reset_tiles(dg2_ctx* c) {
   if (c->d.qm)
     CU(cudaMemsetAsync(c->d.qm, 0xff, 3 * (size_t)c->d.qplane * sizeof(unsigned), c->st));
   launch_finalize(c, 1);
-  return launch_check(c, 2);
+  return launch_check(c, finalize_kernels(c));
 }
 
 int reset_ledger(dg2_ctx* c) {
@@ -772,7 +780,7 @@ int dg2_step(dg2_ctx* c, double dt, double* dt_taken) {
   if ((r = check_not_poisoned(c))) return r;
   dg2::begin_step_kernel<<<1, 1, 0, c->st>>>(c->d, dt);
   enqueue_step(c, true);
-  if ((r = launch_check(c, c->fp32 ? 5 : 6))) return r;
+  if ((r = launch_check(c, 1 + step_kernels(c)))) return r;
   if (dt_taken) {
     Scalars s;
     if ((r = read_scalars(c, &s))) return r;
@@ -821,7 +829,7 @@ int dg2_run_to(dg2_ctx* c, double t_end, int64_t* steps_taken) {
       for (int k = 0; k < chunk; ++k) enqueue_step(c);
       if ((r = launch_check(c, 0))) return r;
     }
-    c->launches += (c->fp32 ? 4 : 5) * (int64_t)chunk;
+    c->launches += step_kernels(c) * (int64_t)chunk;
     if ((r = read_scalars(c, &s))) return r;
     if (s.nonfinite) return fail(DG2_E_NONFINITE, "non-finite state or step near t=%g", s.t);
     if (s.done) break;

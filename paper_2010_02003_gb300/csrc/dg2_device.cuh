@@ -1407,7 +1407,9 @@ static __global__ void __launch_bounds__(TX* TY, 2 * TW / TX) stage_kernel(Dev d
 // ---------------------------------------------------------------------------
 // End of step: one block of kFinThreads threads
 // ---------------------------------------------------------------------------
-constexpr int kFinThreads = 1024;
+// (256: an FP64 sum over more threads costs more on the FP64 pipe than it saves in loads;
+// with 1024 the kernel took 7.7 us on a 128 x 128 grid, FIN_US with 256.)
+constexpr int kFinThreads = 256;
 
 // Builds the next step's tile lists from the non-quiescence flags and the
 // forced mask: a tile is computed if its 3 x 3 tile neighbourhood holds a
@@ -1419,6 +1421,20 @@ constexpr int kFinThreads = 1024;
 // bpart slot and flag, and the step's reductions are exact (max) or summed
 // per tile in a fixed order, so the step's result does not depend on it.
 constexpr int LTX = 32, LTY = 8;
+
+// Weight class of a computed tile: its count of non-quiescent cells (the DG2 cell masks of
+// the new state) in kListClasses equal parts of the tile, the fullest part first.
+__device__ __forceinline__ int weight_class(const Dev& d, int bx, int by) {
+  if (!d.qm || d.scheme != 0) return kListClasses - 1;
+  int nq = 0;
+#pragma unroll
+  for (int yy = 0; yy < TBY; ++yy)
+#pragma unroll
+    for (int xx = 0; xx < TW / WX; ++xx)
+      nq += __popc(d.qm[(long long)(by * TBY + yy) * d.nbx + bx * (TW / WX) + xx]);
+  return kListClasses - 1 - nq * kListClasses / (TW * TY + 1);
+}
+
 static __global__ void __launch_bounds__(LTX* LTY) lists_kernel(Dev d) {
   Scalars* sc = d.sc;
   if (sc->skip_lists) return;
@@ -1464,17 +1480,7 @@ static __global__ void __launch_bounds__(LTX* LTY) lists_kernel(Dev d) {
     if (a) f = false;
     T.act[t] = a ? 1 : 0;
   }
-  // weight class of a computed tile: its count of non-quiescent cells (the DG2
-  // cell masks of the new state) in kListClasses equal parts of the tile, the
-  // fullest part first
-  int cls = kListClasses - 1;
-  if (a && d.qm && d.scheme == 0) {
-    int nq = 0;
-    for (int yy = 0; yy < TBY; ++yy)
-      for (int xx = 0; xx < TW / WX; ++xx)
-        nq += __popc(d.qm[(long long)(by * TBY + yy) * d.nbx + bx * (TW / WX) + xx]);
-    cls = kListClasses - 1 - nq * kListClasses / (TW * TY + 1);
-  }
+  const int cls = a ? weight_class(d, bx, by) : kListClasses - 1;
   // warp = one row of LTX tiles: ballot prefix in the warp, warp offsets, one
   // atomic per class
   const int lane = tid & 31;
@@ -1550,7 +1556,7 @@ static __device__ double ring_inflow(const D& d) {
 // Time, ledger, gauges and the next step; opens the next step's tile lists
 // (built by lists_kernel).  `lists_only`: after a new DEM / state / forced
 // mask, only open the lists.
-static __global__ void __launch_bounds__(kFinThreads) finalize_kernel(Dev d, int lists_only) {
+static __device__ void finalize_body(const Dev& d, int lists_only) {
   Scalars* sc = d.sc;
   if (!lists_only) {
     if (sc->done) {
@@ -1600,6 +1606,68 @@ static __global__ void __launch_bounds__(kFinThreads) finalize_kernel(Dev d, int
     }
   }
   if (threadIdx.x == 0) open_lists(sc);
+}
+
+static __global__ void __launch_bounds__(kFinThreads) finalize_kernel(Dev d, int lists_only) {
+  finalize_body(d, lists_only);
+}
+
+// End of step and the next step's lists in one launch of one block, for grids of up to
+// kSmallTiles tiles (the rules of lists_kernel; entries take their places from counters in
+// shared memory).  A launch and its gap were a tenth of a step there.
+constexpr int kSmallTiles = 1024;
+static __global__ void __launch_bounds__(kFinThreads) finalize_small_kernel(Dev d, int lists_only) {
+  finalize_body(d, lists_only);
+  __shared__ unsigned char busy[kSmallTiles];
+  __shared__ int cnt[kListClasses + 1], skip;
+  Scalars* sc = d.sc;
+  const Tiles& T = d.tiles;
+  const int ntx = T.ntx, nty = T.nty, nt = T.ntiles, tid = threadIdx.x;
+  if (tid == 0) skip = sc->skip_lists;
+  if (tid <= kListClasses) cnt[tid] = 0;
+  const bool every = !T.skip || T.all_forced;
+  for (int t = tid; t < nt && !every; t += kFinThreads) {
+    unsigned char v = T.forced[t];
+    for (int k = 0; k < d.nsub; ++k) v |= T.flag[t * d.nsub + k];
+    busy[t] = v != 0;
+  }
+  __syncthreads();
+  if (skip) return;
+  for (int t = tid; t < nt; t += kFinThreads) {
+    if (every) {
+      T.act[t] = 1;
+      continue;
+    }
+    const int bx = t % ntx, by = t / ntx;
+    bool a = false, f = false;
+#pragma unroll
+    for (int oy = -2; oy <= 2; ++oy)
+#pragma unroll
+      for (int ox = -2; ox <= 2; ++ox) {
+        const int x = bx + ox, y = by + oy;
+        if (x < 0 || y < 0 || x >= ntx || y >= nty || !busy[y * ntx + x]) continue;
+        if (ox >= -1 && ox <= 1 && oy >= -1 && oy <= 1) a = true;
+        else f = true;
+      }
+    T.act[t] = a ? 1 : 0;
+    if (a) {
+      const int cls = weight_class(d, bx, by);
+      T.list[cls * nt + atomicAdd(&cnt[cls], 1)] = t;
+    } else if (f) {
+      T.front[atomicAdd(&cnt[kListClasses], 1)] = t;
+    }
+  }
+  __syncthreads();
+  if (tid == 0) {
+    int n = 0;
+    for (int k = 0; k < kListClasses; ++k) {
+      sc->n_b[k] = cnt[k];
+      n += cnt[k];
+    }
+    sc->n_act = every ? nt : n;
+    sc->n_front = cnt[kListClasses];
+    sc->list_all = every ? 1 : 0;
+  }
 }
 
 // Uploaded state (dg2_set_state): nine dense FP64 planes staged in T.  The check writes
