@@ -980,13 +980,10 @@ int dg2_set_state(dg2_ctx* c, const double* planes, double t) {
   Scalars s;
   if ((r = read_scalars(c, &s))) return r;
   if (first != ~0ull) return fail(DG2_E_ARG, "non-finite state value %llu", first);
-  if (c->fp32) {
-    CU(cudaMemcpyAsync(c->f.S, c->f.T, dg2::f32::kPlanes32 * (size_t)c->f.plane * sizeof(float),
-                       cudaMemcpyDeviceToDevice, c->st));
-  } else {
-    dg2::state_in_kernel<<<c->pgrid, c->pblock, 0, c->st>>>(c->d);
-    if ((r = launch_check(c, 1))) return r;
-  }
+  // the state, with the flags (and cell masks) of what in it is not still and dry
+  if (c->fp32) dg2::f32::state_commit32_kernel<<<c->pgrid, c->pblock, 0, c->st>>>(c->f, tile_w(c));
+  else dg2::state_in_kernel<<<c->pgrid, c->pblock, 0, c->st>>>(c->d);
+  if ((r = launch_check(c, 1))) return r;
   s.t = t;
   s.done = 0;
   s.nonfinite = 0;
@@ -997,7 +994,8 @@ int dg2_set_state(dg2_ctx* c, const double* planes, double t) {
   s.ledger_init = 1;  // the mass kernel below resets the ledger
   CU(cudaMemcpyAsync(c->d.sc, &s, sizeof s, cudaMemcpyHostToDevice, c->st));
   c->dem_set = 1;
-  if ((r = reset_tiles(c))) return r;
+  launch_finalize(c, 1);  // the next step's lists
+  if ((r = launch_check(c, finalize_kernels(c)))) return r;
   launch_mass(c);
   if ((r = launch_check(c, 1))) return r;
   if ((r = recompute_dt(c))) return r;

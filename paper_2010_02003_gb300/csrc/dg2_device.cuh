@@ -1407,9 +1407,23 @@ static __global__ void __launch_bounds__(TX* TY, 2 * TW / TX) stage_kernel(Dev d
 // ---------------------------------------------------------------------------
 // End of step: one block of kFinThreads threads
 // ---------------------------------------------------------------------------
-// (256: an FP64 sum over more threads costs more on the FP64 pipe than it saves in loads;
-// with 1024 the kernel took 7.7 us on a 128 x 128 grid, FIN_US with 256.)
+// The block works on a copy of the scalars in shared memory, read and written back in one
+// access per thread: thread 0's walk through them in global memory was a chain of round
+// trips to L2, a good part of the kernel (2000 x 1000 cells: 8.7 us, 7.6 now).  256
+// threads: an FP64 sum over more costs more on the FP64 pipe than it saves in loads.
 constexpr int kFinThreads = 256;
+
+__device__ __forceinline__ void scalars_in(Scalars* to, const Scalars* from) {
+  static_assert(sizeof(Scalars) % 8 == 0 && sizeof(Scalars) / 8 <= kFinThreads, "one word a thread");
+  if (threadIdx.x < sizeof(Scalars) / 8)
+    reinterpret_cast<long long*>(to)[threadIdx.x] = reinterpret_cast<const long long*>(from)[threadIdx.x];
+  __syncthreads();
+}
+__device__ __forceinline__ void scalars_out(Scalars* to, const Scalars* from) {
+  __syncthreads();
+  if (threadIdx.x < sizeof(Scalars) / 8)
+    reinterpret_cast<long long*>(to)[threadIdx.x] = reinterpret_cast<const long long*>(from)[threadIdx.x];
+}
 
 // Builds the next step's tile lists from the non-quiescence flags and the
 // forced mask: a tile is computed if its 3 x 3 tile neighbourhood holds a
@@ -1556,8 +1570,7 @@ static __device__ double ring_inflow(const D& d) {
 // Time, ledger, gauges and the next step; opens the next step's tile lists
 // (built by lists_kernel).  `lists_only`: after a new DEM / state / forced
 // mask, only open the lists.
-static __device__ void finalize_body(const Dev& d, int lists_only) {
-  Scalars* sc = d.sc;
+static __device__ void finalize_body(const Dev& d, Scalars* sc, int lists_only) {
   if (!lists_only) {
     if (sc->done) {
       if (threadIdx.x == 0) sc->skip_lists = 1;
@@ -1609,7 +1622,10 @@ static __device__ void finalize_body(const Dev& d, int lists_only) {
 }
 
 static __global__ void __launch_bounds__(kFinThreads) finalize_kernel(Dev d, int lists_only) {
-  finalize_body(d, lists_only);
+  __shared__ Scalars sc;
+  scalars_in(&sc, d.sc);
+  finalize_body(d, &sc, lists_only);
+  scalars_out(d.sc, &sc);
 }
 
 // End of step and the next step's lists in one launch of one block, for grids of up to
@@ -1617,13 +1633,13 @@ static __global__ void __launch_bounds__(kFinThreads) finalize_kernel(Dev d, int
 // shared memory).  A launch and its gap were a tenth of a step there.
 constexpr int kSmallTiles = 1024;
 static __global__ void __launch_bounds__(kFinThreads) finalize_small_kernel(Dev d, int lists_only) {
-  finalize_body(d, lists_only);
+  __shared__ Scalars sc;
   __shared__ unsigned char busy[kSmallTiles];
-  __shared__ int cnt[kListClasses + 1], skip;
-  Scalars* sc = d.sc;
+  __shared__ int cnt[kListClasses + 1];
+  scalars_in(&sc, d.sc);
+  finalize_body(d, &sc, lists_only);
   const Tiles& T = d.tiles;
   const int ntx = T.ntx, nty = T.nty, nt = T.ntiles, tid = threadIdx.x;
-  if (tid == 0) skip = sc->skip_lists;
   if (tid <= kListClasses) cnt[tid] = 0;
   const bool every = !T.skip || T.all_forced;
   for (int t = tid; t < nt && !every; t += kFinThreads) {
@@ -1632,7 +1648,10 @@ static __global__ void __launch_bounds__(kFinThreads) finalize_small_kernel(Dev 
     busy[t] = v != 0;
   }
   __syncthreads();
-  if (skip) return;
+  if (sc.skip_lists) {  // the step was not taken
+    scalars_out(d.sc, &sc);
+    return;
+  }
   for (int t = tid; t < nt; t += kFinThreads) {
     if (every) {
       T.act[t] = 1;
@@ -1661,13 +1680,14 @@ static __global__ void __launch_bounds__(kFinThreads) finalize_small_kernel(Dev 
   if (tid == 0) {
     int n = 0;
     for (int k = 0; k < kListClasses; ++k) {
-      sc->n_b[k] = cnt[k];
+      sc.n_b[k] = cnt[k];
       n += cnt[k];
     }
-    sc->n_act = every ? nt : n;
-    sc->n_front = cnt[kListClasses];
-    sc->list_all = every ? 1 : 0;
+    sc.n_act = every ? nt : n;
+    sc.n_front = cnt[kListClasses];
+    sc.list_all = every ? 1 : 0;
   }
+  scalars_out(d.sc, &sc);
 }
 
 // Uploaded state (dg2_set_state): nine dense FP64 planes staged in T.  The check writes
@@ -1686,12 +1706,37 @@ static __global__ void __launch_bounds__(256) state_check_kernel(Dev d, unsigned
       return;
     }
 }
+// One block per 32 x 8 tile.  The copy also writes the tiles' flags and the cell masks of the
+// new state, so the first step leaves still, dry ground out as every other does (computing
+// the whole grid there was a twentieth of a pass of 84 steps of a 2000 x 1000 floodplain).
+// A cell below -1 m counts as moving: the first step then meets its check.
 static __global__ void __launch_bounds__(256) state_in_kernel(Dev d) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
-  if (i >= d.nx || j >= d.ny) return;
-  const long long n = (long long)d.nx * d.ny, c = (long long)j * d.nx + i;
+  __shared__ int moving[TW / WX];
+  const int tid = threadIdx.y * TW + threadIdx.x, lane = tid & 31;
+  int cx, cy;
+  warp_cell<TW>(cx, cy);
+  if (tid < TW / WX) moving[tid] = 0;
+  __syncthreads();
+  const int i = blockIdx.x * TW + cx, j = blockIdx.y * TY + cy;
+  bool nq = false;
+  if (i < d.nx && j < d.ny) {
+    const long long n = (long long)d.nx * d.ny, c = (long long)j * d.nx + i;
 #pragma unroll
-  for (int k = 0; k < 9; ++k) d.S[k * d.plane + (long long)j * d.pitch + i] = d.T[k * n + c];
+    for (int k = 0; k < 9; ++k) {
+      const double v = d.T[k * n + c];
+      d.S[k * d.plane + (long long)j * d.pitch + i] = v;
+      if (k == 0) nq = above(v, d.tol) || v < -1.0;
+      else if (d.scheme == 0 || k % 3 == 0) nq = nq || nonzero(v);
+    }
+  }
+  const unsigned bits = __ballot_sync(0xffffffffu, nq);
+  if (lane == 0) {
+    if (d.qm)
+      d.qm[(long long)(blockIdx.y * TBY + cy / WY) * d.nbx + blockIdx.x * (TW / WX) + cx / WX] = bits;
+    if (bits) moving[cx / WX * d.nsub / (TW / WX)] = 1;
+  }
+  __syncthreads();
+  if (tid < d.nsub) d.tiles.flag[(blockIdx.y * d.tiles.ntx + blockIdx.x) * d.nsub + tid] = moving[tid];
 }
 
 // Courant reduction of the current state alone (after set-up or set_state).

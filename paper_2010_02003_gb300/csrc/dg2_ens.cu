@@ -176,13 +176,14 @@ __global__ void __launch_bounds__(BX* BY, BX * BY <= 128 ? 2 * DG2_MINB32 : DG2_
 // member's next dt; counts members that reach t_end; opens the next lists.
 __global__ void __launch_bounds__(kFinThreads) ens_finalize_kernel(EnsDev E, int lists_only) {
   const D32& d = E.desc[blockIdx.x];
-  __shared__ int was_done;
-  if (threadIdx.x == 0) was_done = d.sc->done;
+  __shared__ Scalars sc;
+  scalars_in(&sc, d.sc);
+  const int was_done = sc.done;
   __syncthreads();
-  f32::finalize32_body(d, lists_only);
-  __syncthreads();
-  if (threadIdx.x == 0 && !lists_only && !was_done && d.sc->done) atomicAdd(&E.es->n_done, 1);
-  if (threadIdx.x == 0 && d.sc->nonfinite) E.es->bad = 1;
+  f32::finalize32_body(d, &sc, lists_only);
+  scalars_out(d.sc, &sc);
+  if (threadIdx.x == 0 && !lists_only && !was_done && sc.done) atomicAdd(&E.es->n_done, 1);
+  if (threadIdx.x == 0 && sc.nonfinite) E.es->bad = 1;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     E.es->n_act = 0;
     E.es->n_front = 0;

@@ -439,8 +439,7 @@ struct Blk32 {
 
 // Time, ledger, gauges and the next step; opens the next step's tile lists.
 // Run by one block of kFinThreads threads per problem.
-static __device__ void finalize32_body(const D32& d, int lists_only) {
-  Scalars* sc = d.sc;
+static __device__ void finalize32_body(const D32& d, Scalars* sc, int lists_only) {
   if (!lists_only) {
     if (sc->done) {
       if (threadIdx.x == 0) sc->skip_lists = 1;
@@ -543,6 +542,36 @@ static __global__ void __launch_bounds__(256) state_in32_kernel(D32 d, const dou
     d.T[k * P + o] = f;
     if (k == 0) d.T[E0L * P + o] = to_f32(v - to_f64(f));
   }
+}
+
+// The checked state from T to S, with the flags of the tiles (tw x 8 cells, 16 or 32 wide)
+// that hold a cell which is not still and dry, so the first step leaves the others out as
+// every step does.  One block per 32 x 8 cells.
+static __global__ void __launch_bounds__(256) state_commit32_kernel(D32 d, int tw) {
+  __shared__ int moving[2];
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
+  const int tid = threadIdx.y * 32 + threadIdx.x;
+  if (tid < 2) moving[tid] = 0;
+  __syncthreads();
+  bool nq = false;
+  if (i < d.nx && j < d.ny) {
+    const long long P = d.plane, o = (long long)j * d.pitch + i;
+    float m[kPlanes32];
+#pragma unroll
+    for (int k = 0; k < kPlanes32; ++k) {
+      m[k] = d.T[k * P + o];
+      d.S[k * P + o] = m[k];
+    }
+    float z0, z1x, z1y, zE, zW, zN, zS;
+    cell_z(d, i, j, z0, z1x, z1y, zE, zW, zN, zS);
+    nq = !((m[E0] - z0) + m[E0L] <= d.tol) || m[E1X] != z1x || m[E1Y] != z1y;
+#pragma unroll
+    for (int k = 3; k < 9; ++k) nq = nq || m[k] != 0.f;
+  }
+  if (nq) moving[threadIdx.x / tw] = 1;
+  __syncthreads();
+  const int t = blockIdx.x * (32 / tw) + tid;
+  if (tid < 32 / tw && t < d.tiles.ntx) d.tiles.flag[blockIdx.y * d.tiles.ntx + t] = moving[tid];
 }
 
 // Planes k0 .. k0 + m - 1 of the state as dense FP64 depth modes.
