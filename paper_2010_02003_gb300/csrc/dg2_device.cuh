@@ -448,9 +448,10 @@ __device__ __forceinline__ double minmod3(double a, double b, double c) {
 
 // Detector (Eq. 6, tested as J > thresh * den, the magnitude in den floored at
 // tol_dry) and generalised minmod (Eq. 7) for one component along one direction.
-__device__ __forceinline__ double limit_component(double thresh, double tol, double half,
-                                                  double k0w, double k1w, double k0, double k1,
-                                                  double k0e, double k1e) {
+// `th` is the threshold times half the cell size.
+__device__ __forceinline__ double limit_component(double th, double tol, double k0w,
+                                                  double k1w, double k0, double k1, double k0e,
+                                                  double k1e) {
   // k1 / sqrt(3) as a product with 1 / sqrt(3) rounded to nearest (one FP64
   // division fewer per component; within an ulp of the quotient)
   const double q = k1 * 0.57735026918962576;
@@ -460,10 +461,33 @@ __device__ __forceinline__ double limit_component(double thresh, double tol, dou
   // share a sign, a sum of magnitudes, rounded alike
   double mag = fabs(k0) + fabs(q);
   if (fbits(mag) < fbits(tol)) mag = tol;  // still water: round-off never counts as a shock
-  const double den = half * mag;
   const double jm = max_nn(jE, jW);
-  if (!gt(jm, thresh * den)) return k1;
+  if (!gt(jm, th * mag)) return k1;
   return minmod3(k1, k0e - k0, k0 - k0w);
+}
+
+// x cut to FP32 on the integer units: towards zero, 0 below 2^-126, infinite from 2^128 on.
+__device__ __forceinline__ float cut32(double x) {
+  const int hi = __double2hiint(x), e = hi & 0x7fffffff;
+  const float f = __int_as_float((hi & 0x80000000) | ((e - 0x38000000) << 3) |
+                                 (int)((unsigned)__double2loint(x) >> 29));
+  return e < 0x38100000 ? 0.f : e >= 0x47f00000 ? __int_as_float(0x7f800000) : f;
+}
+
+// Whether limit_component certainly finds no shock, by the same test in FP32.  Jumps are
+// rarely a hundredth of Eq. 6's threshold, and FP32 arithmetic is 64 times cheaper here than
+// the nine FP64 operations of the test.  The values are cut within 2^-23 of their
+// magnitudes, so with s the sum of the magnitudes of all terms jumps and threshold are off
+// by less than 2^-20 s and 2^-20 th s; the margin is four times that, and 1e-36 for values
+// that FP32 flushes.  Not certain (or not
+// finite): the FP64 test decides, so the slopes do not depend on this one.  DG2-LL stages,
+// without -> with it: 1000 x 600 flooded plain 541 / 598 -> 387 / 450 us, 2000 x 1000
+// floodplain 87 / 96 -> 75 / 83 us.
+__device__ __forceinline__ bool calm(float th, float tol, float k0w, float k1w, float k0, float k1,
+                                     float k0e, float k1e, float s) {
+  const float jE = fabsf((k0e - k1e) - (k0 + k1)), jW = fabsf((k0 - k1) - (k0w + k1w));
+  const float mag = fmaxf(fabsf(k0) + 0.57735f * fabsf(k1), tol);
+  return fmaxf(jE, jW) + 4e-6f * s * (1.f + th) + 1e-36f < 0.9999f * (th * mag);
 }
 
 // Slopes (h, qx, qy) of cell (i, j) along `dir` (1 = x, 2 = y) from buffer U,
@@ -483,22 +507,32 @@ static __device__ void limited_slopes(const Dev& d, const double* __restrict__ U
   const long long ch = dir == 1 ? c + 1 : c + d.pitch;
   const double hl = U[cl], hc = U[c], hh = U[ch];
   if (!above(hl, d.tol) || !above(hc, d.tol) || !above(hh, d.tol)) return;
-  const double half = 0.5 * (dir == 1 ? d.dx : d.dy);
-  const double* z0 = d.Z;
-  const double* z1 = d.Z + dir * P;
-  const double e1c = sh + z1[c];
-  const double e1 = limit_component(d.ds, d.tol, half, hl + z0[cl], U[dir * P + cl] + z1[cl],
-                                    hc + z0[c], e1c, hh + z0[ch], U[dir * P + ch] + z1[ch]);
-  if (e1 != e1c) sh = e1 - z1[c];
+  const double th = d.ds * 0.5 * (dir == 1 ? d.dx : d.dy);
+  const float thf = cut32(d.ds) * 0.5f * cut32(dir == 1 ? d.dx : d.dy), tolf = cut32(d.tol);
+  const double *z0 = d.Z, *z1 = d.Z + dir * P, *h1 = U + dir * P;
   {
-    const double* k0 = U + 3 * P;
-    const double* k1 = U + (3 + dir) * P;
-    sqx = limit_component(d.ds, d.tol, half, k0[cl], k1[cl], k0[c], k1[c], k0[ch], k1[ch]);
+    const float al = cut32(hl), ac = cut32(hc), ah = cut32(hh);
+    const float bl = cut32(z0[cl]), bc = cut32(z0[c]), bh = cut32(z0[ch]);
+    const float sl = cut32(h1[cl]), sc = cut32(sh), s2 = cut32(h1[ch]);
+    const float tl = cut32(z1[cl]), tc = cut32(z1[c]), t2 = cut32(z1[ch]);
+    const float s = fabsf(al) + fabsf(ac) + fabsf(ah) + fabsf(bl) + fabsf(bc) + fabsf(bh) +
+                    fabsf(sl) + fabsf(sc) + fabsf(s2) + fabsf(tl) + fabsf(tc) + fabsf(t2);
+    if (!calm(thf, tolf, al + bl, sl + tl, ac + bc, sc + tc, ah + bh, s2 + t2, s)) {
+      const double e1c = sh + z1[c];
+      const double e1 = limit_component(th, d.tol, hl + z0[cl], h1[cl] + z1[cl], hc + z0[c], e1c,
+                                        hh + z0[ch], h1[ch] + z1[ch]);
+      if (fbits(e1) != fbits(e1c)) sh = e1 - z1[c];  // (limited)
+    }
   }
-  {
-    const double* k0 = U + 6 * P;
-    const double* k1 = U + (6 + dir) * P;
-    sqy = limit_component(d.ds, d.tol, half, k0[cl], k1[cl], k0[c], k1[c], k0[ch], k1[ch]);
+#pragma unroll
+  for (int v = 1; v <= 2; ++v) {
+    const double *k0 = U + 3 * v * P, *k1 = U + (3 * v + dir) * P;
+    double& sq = v == 1 ? sqx : sqy;
+    const float a = cut32(k0[cl]), b = cut32(k1[cl]), e = cut32(k0[c]), f = cut32(sq);
+    const float g = cut32(k0[ch]), h = cut32(k1[ch]);
+    const float s = fabsf(a) + fabsf(b) + fabsf(e) + fabsf(f) + fabsf(g) + fabsf(h);
+    if (!calm(thf, tolf, a, b, e, f, g, h, s))
+      sq = limit_component(th, d.tol, k0[cl], k1[cl], k0[c], k1[c], k0[ch], k1[ch]);
   }
 }
 
