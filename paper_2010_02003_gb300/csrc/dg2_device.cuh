@@ -480,9 +480,9 @@ __device__ __forceinline__ float cut32(double x) {
 // magnitudes, so with s the sum of the magnitudes of all terms jumps and threshold are off
 // by less than 2^-20 s and 2^-20 th s; the margin is four times that, and 1e-36 for values
 // that FP32 flushes.  Not certain (or not
-// finite): the FP64 test decides, so the slopes do not depend on this one.  DG2-LL stages,
-// without -> with it: 1000 x 600 flooded plain 541 / 598 -> 387 / 450 us, 2000 x 1000
-// floodplain 87 / 96 -> 75 / 83 us.
+// finite): the FP64 test decides, so the slopes do not depend on this one.  Without -> with
+// it: 2000 x 1000 floodplain, stages 87 / 96 -> 75 / 83 us; 1000 x 600 flooded plain, pass of
+// 33 steps 41.9 -> 34.1 ms (stages 387 / 450 us with it).
 __device__ __forceinline__ bool calm(float th, float tol, float k0w, float k1w, float k0, float k1,
                                      float k0e, float k1e, float s) {
   const float jE = fabsf((k0e - k1e) - (k0 + k1)), jW = fabsf((k0 - k1) - (k0w + k1w));
