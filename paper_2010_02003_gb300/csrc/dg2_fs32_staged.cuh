@@ -14,10 +14,13 @@
 // flux per face, the operator of Eqs. 4-5 and the RK update.
 //
 // Friction (Sec. 2.1.3, implicit splitting once per step before stage 1) is
-// applied here instead of in a pass of its own: stage 1 applies it to every
-// staged cell in shared memory before anything else reads them (a cell's
-// friction depends on that cell alone, so the halo cells of a tile get exactly
-// the values their own tile computes).  Stage 2 needs the post-friction U^n
+// applied here instead of in a pass of its own (a cell's friction depends on that
+// cell alone, so the halo cells of a tile get exactly the values their own tile
+// computes).  DG2-LL stage 1 applies it to every staged cell in shared memory before
+// anything else reads them; DG2-NL stage 1, where a cell's discharges are read by its own
+// thread and, in the halo, by the one thread that builds its record, to registers
+// there, without the pass and its barrier (2000 x 1000 flooded plain, stage 1 122 -> 116
+// us; 2900 x 2900 urban grid 499 -> 469 us; the same bits).  Stage 2 needs the post-friction U^n
 // for the RK average: in DG2-NL stage 1 stores its own cells' six discharge
 // modes after friction in Q (stage 2 reads them in place of U^n's, so it
 // evaluates no friction); in DG2-LL, whose Q holds the limited slopes of U^n,
@@ -209,19 +212,38 @@ __device__ __forceinline__ void staged_limited(const D32& d, const SM& sm, int r
   sqy = limit_comp32(d.ds, d.tol, half, k0[cl], k1[cl], k0[c], k1[c], k0[ch], k1[ch]);
 }
 
+// Discharge modes of the staged cell (r, x), in the order of the planes, after friction when
+// the stage has not applied it to the staged planes (`rub`: DG2-NL stage 1).
+template <bool RUB, int SP, class SM>
+__device__ __forceinline__ void staged_discharge(const SM& sm, int r, int x, float gdt, float tol,
+                                                 float q[6]) {
+  const int c = r * SP + x;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) q[k] = sm.st.u[QX0 + k][c];
+  if (RUB) {
+    float z0, z1x, z1y, zE, zW, zN, zS;
+    staged_z(sm, r, x, z0, z1x, z1y, zE, zW, zN, zS);
+    const float h0 = (sm.st.u[E0][c] - z0) + sm.st.u[E0L][c];
+    friction_modes32(gdt, sm.st.n[c], tol, h0, sm.st.u[E1X][c] - z1x, sm.st.u[E1Y][c] - z1y, q);
+  }
+}
+
 // Planar limit (face depth, qx, qy) of the staged cell (r, x) at face f (0 E,
 // 1 W, 2 N, 3 S), slopes limited when LL: for an edge ghost.
-template <bool LL, int SP, class SM>
+template <bool LL, bool RUB, int SP, class SM>
 __device__ __forceinline__ void staged_face_limit(const D32& d, const SM& sm, int r, int x, int gi,
-                                                  int gj, int f, float& h, float& qx, float& qy) {
+                                                  int gj, int f, float gdt, float& h, float& qx,
+                                                  float& qy) {
   const int c = r * SP + x;
   const int dir = f <= 1 ? 1 : 2;
-  float se = sm.st.u[dir][c], sx = sm.st.u[3 + dir][c], sy = sm.st.u[6 + dir][c];
+  float q[6];
+  staged_discharge<RUB, SP>(sm, r, x, gdt, d.tol, q);
+  float se = sm.st.u[dir][c], sx = dir == 1 ? q[1] : q[2], sy = dir == 1 ? q[4] : q[5];
   if (LL) staged_limited<SP>(d, sm, r, x, gi, gj, dir, se, sx, sy);
   float z0, z1x, z1y, zE, zW, zN, zS;
   staged_z(sm, r, x, z0, z1x, z1y, zE, zW, zN, zS);
   const float e0 = sm.st.u[E0][c], lo = sm.st.u[E0L][c];
-  const float x0 = sm.st.u[QX0][c], y0 = sm.st.u[QY0][c];
+  const float x0 = q[0], y0 = q[3];
   if (f == 0) { h = ((e0 - zE) + se) + lo; qx = x0 + sx; qy = y0 + sy; }
   else if (f == 1) { h = ((e0 - zW) - se) + lo; qx = x0 - sx; qy = y0 - sy; }
   else if (f == 2) { h = ((e0 - zN) + se) + lo; qx = x0 + sx; qy = y0 + sy; }
@@ -231,12 +253,14 @@ __device__ __forceinline__ void staged_face_limit(const D32& d, const SM& sm, in
 // Record of the staged neighbour (r, x) = grid (gi, gj) at the face it shares
 // with a tile cell (side 0: west / south of the face, its east / north limit;
 // side 1: east / north, its west / south limit) along dir.
-template <bool LL, int SP, class SM>
+template <bool LL, bool RUB, int SP, class SM>
 __device__ __forceinline__ RecF staged_neighbour_rec(const D32& d, const SM& sm, int r, int x,
-                                                     int gi, int gj, int dir, int side) {
+                                                     int gi, int gj, int dir, int side, float gdt) {
   const int c = r * SP + x;
-  float ex = sm.st.u[E1X][c], xx = sm.st.u[QX1X][c], yx = sm.st.u[QY1X][c];
-  float ey = sm.st.u[E1Y][c], xy = sm.st.u[QX1Y][c], yy = sm.st.u[QY1Y][c];
+  float q[6];
+  staged_discharge<RUB, SP>(sm, r, x, gdt, d.tol, q);
+  float ex = sm.st.u[E1X][c], xx = q[1], yx = q[4];
+  float ey = sm.st.u[E1Y][c], xy = q[2], yy = q[5];
   if (LL) {
     staged_limited<SP>(d, sm, r, x, gi, gj, 1, ex, xx, yx);
     staged_limited<SP>(d, sm, r, x, gi, gj, 2, ey, xy, yy);
@@ -249,7 +273,7 @@ __device__ __forceinline__ RecF staged_neighbour_rec(const D32& d, const SM& sm,
   float scl;
   const float h0 = (e0 - z0) + lo;
   const bool pw = pw_scale32(h0, wh, eh, sh, nh, d.tol, d.wd, scl);
-  const float qx0 = sm.st.u[QX0][c], qy0 = sm.st.u[QY0][c];
+  const float qx0 = q[0], qy0 = q[3];
   const bool thin = d.wd != 0;
   // the limit at the shared face, selected (one record built whatever dir and side)
   const float hf = dir == 1 ? (side == 0 ? eh : wh) : (side == 0 ? nh : sh);
@@ -360,8 +384,11 @@ __device__ __forceinline__ void stage32_staged(const D32& d, StagedSmem32<LL, ST
     __syncthreads();
   }
 
-  // ---- stage 1: friction of every staged cell the stage reads, in place ----
-  if (STAGE == 1) {
+  // ---- stage 1: friction.  DG2-LL, whose limiter reads neighbours, applies it to every
+  // staged cell in place; DG2-NL to a cell's registers where it is read (its own thread, and
+  // the thread of its record beyond the tile): no pass of its own and no barrier. ----
+  constexpr bool RUB = STAGE == 1 && !LL;
+  if (STAGE == 1 && LL) {
     constexpr int RW = BX + 2 * H;
     for (int k = tid; k < SR * RW; k += NT) {
       const int r = k / RW, cc = k - r * RW;
@@ -395,6 +422,9 @@ __device__ __forceinline__ void stage32_staged(const D32& d, StagedSmem32<LL, ST
       staged_limited<SP>(d, sm, r0, x0, i, j, 2, m[E1Y], m[QX1Y], m[QY1Y]);
     }
     staged_z(sm, r0, x0, z0, z1x, z1y, zE, zW, zN, zS);
+    if (RUB)
+      friction_modes32(gdt, sm.st.n[STAGE == 1 ? c0 : 0], tol, (m[E0] - z0) + mlo, m[E1X] - z1x,
+                       m[E1Y] - z1y, m + QX0);
     float eh, wh, nh, shh;
     face_depths32(m[E0], m[E1X], m[E1Y], mlo, zE, zW, zN, zS, eh, wh, nh, shh);
     const float eqx = m[QX0] + m[QX1X], eqy = m[QY0] + m[QY1X];
@@ -436,12 +466,12 @@ __device__ __forceinline__ void stage32_staged(const D32& d, StagedSmem32<LL, ST
         // the ghost of the tile cell's own limit at that face
         const int fo = kind == 0 ? 1 : kind == 1 ? 0 : kind == 2 ? 3 : 2;
         float h, qx, qy;
-        staged_face_limit<LL, SP>(d, sm, r, x, gi, gj, fo, h, qx, qy);
+        staged_face_limit<LL, RUB, SP>(d, sm, r, x, gi, gj, fo, gdt, h, qx, qy);
         const float s = dir == 1 ? (gj + 0.5f) * d.dy : (gi + 0.5f) * d.dx;
         ghost32(d, kind, s, ts, h, qx, qy);
         rec = make_rec32(h, qx, qy, false, 1.f, tol);
       } else {
-        rec = staged_neighbour_rec<LL, SP>(d, sm, r + sy, x + sx, gi + sx, gj + sy, dir, side);
+        rec = staged_neighbour_rec<LL, RUB, SP>(d, sm, r + sy, x + sx, gi + sx, gj + sy, dir, side, gdt);
       }
       RecF* dst = kind == 0 ? sm.hw : kind == 1 ? sm.he : kind == 2 ? sm.hs : sm.hn;
       dst[q] = rec;
