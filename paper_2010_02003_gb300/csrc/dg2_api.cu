@@ -61,7 +61,7 @@ size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 // 250, 265.  So 16 columns, and 8 on grids of up to two tiles per SM.
 constexpr int kFineTiles = 304;
 int parts64(int nx, int ny, int scheme) {
-  if (scheme != DG2_SCHEME_DG2) return 1;
+  if (scheme != DG2_SCHEME_DG2) return dg2::fv::PARTS;
   const long long nt = (long long)((nx + 31) / 32) * ((ny + 7) / 8);
   return nt <= kFineTiles ? 4 : 2;
 }
@@ -319,8 +319,7 @@ void enqueue_step(dg2_ctx* c, bool timed = false) {
   // FP32: friction is fused into the stage kernels (no launch of its own)
   if (!c->fp32) {
     if (d.nsub == 4) dg2::friction_kernel<8><<<c->g_fric, c->sblock, 0, c->st>>>(d);
-    else if (d.nsub == 2) dg2::friction_kernel<16><<<c->g_fric, c->sblock, 0, c->st>>>(d);
-    else dg2::friction_kernel<32><<<c->g_fric, c->sblock, 0, c->st>>>(d);
+    else dg2::friction_kernel<16><<<c->g_fric, c->sblock, 0, c->st>>>(d);
   }
   if (e) cudaEventRecord(e[1], c->st);
   if (c->p.scheme != DG2_SCHEME_DG2) {

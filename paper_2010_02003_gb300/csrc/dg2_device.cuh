@@ -24,7 +24,7 @@ namespace dg2 {
 
 // The tiles of the FP64 lists are TW x TY = 32 x 8 cells.  A block of the DG2 kernels works
 // on a part of one, TX x TY cells (TX a template parameter, TW / TX parts a tile,
-// Dev::nsub; the FV kernels take whole tiles).  A warp covers a WX x WY block of cells
+// Dev::nsub; the FV kernels take halves).  A warp covers a WX x WY block of cells
 // (lane l: column l % WX, row l / WX of the block); a part is TX / 8 x 2 such blocks, warp w
 // the block (w % (TX / 8), w / (TX / 8)).  Wet regions are compact, so square-ish blocks
 // hold fewer dry lanes than rows of 32.  The cell of the calling thread in its part:
@@ -120,7 +120,7 @@ struct Scalars {
 // skip = 0 compute every cell.
 struct Tiles {
   unsigned char* flag;          // [ntiles * parts] part of a tile held a non-quiescent cell
-                                // after the last stage 2 (parts: 1, FP64 DG2 Dev::nsub)
+                                // after the last stage 2 (parts: FP32 1, FP64 Dev::nsub)
   unsigned char* act;           // [ntiles] tile computed in the current step
   const unsigned char* forced;  // [ntiles] tile must be computed (inflow, source); set on the host
   int* list;                    // [kListClasses * ntiles] computed tiles of the step, by weight class
@@ -186,7 +186,7 @@ struct Dev {
   // cells stage 1 computed (plane 2)
   unsigned int* qm;
   int nbx, nby;              // warp blocks per row / column (whole 32 x 8 tiles)
-  int nsub;                  // blocks (parts) per tile: 1, FP64 DG2 2 or 4 (parts64)
+  int nsub;                  // blocks (parts) per tile: FP64 2 or 4 (parts64), FP32 1
   long long qplane;          // words per qm plane
 };
 

@@ -10,7 +10,7 @@
 // Eq. 8's bed term (factor 2 / dx as in Eq. 4a).  Friction is the DG2 friction
 // kernel, which on zero slopes acts on the averages alone.
 //
-// One block per 32 x 8 tile of the step's lists, as the DG2 stage kernels:
+// One block per 16 x 8 half of a tile of the step's lists, as the DG2 stage kernels:
 // the averages of the tile and a 2-cell halo are staged in shared memory, each
 // thread forms its cell's four limits, the tile's last threads form the limits
 // beyond the tile, and every face flux is evaluated once.  Dry-tile skipping
@@ -29,7 +29,7 @@
 namespace dg2 {
 namespace fv {
 
-constexpr int TX = TW;                   // a block takes a whole tile
+constexpr int TX = 16, PARTS = TW / TX;  // a block takes half a tile
 constexpr int HX = TX + 4, HY = TY + 4;  // staged region: tile + 2-cell halo
 
 struct L4 {
@@ -147,14 +147,14 @@ __device__ __forceinline__ Face face(const L4& a, const L4& b, bool ydir, double
   return Face{F.h, F.n, F.t, F.dp, ha};
 }
 
-// One FV stage on the 32 x 8 tile (bx, by).  Stage 1: T = S + dt L(S) (all
+// One FV stage on the 16 x 8 part (bx, by) of tile `tile`.  Stage 1: T = S + dt L(S) (all
 // of FV1's update); stage 2 (FV2): S = (S + T + dt L(T)) / 2.  A dry cell
 // keeps no discharge.  Accumulates the boundary inflow rate, and in the last
 // stage the Courant rate and the non-finite / non-quiescent flags, of the
 // thread's cell.
 template <bool ORDER2, int STAGE>
-__device__ __forceinline__ void fv_tile(const Dev& d, Smem& sm, int bx, int by, double& brate,
-                                        double& lam, bool& bad, bool& nonq) {
+__device__ __forceinline__ void fv_tile(const Dev& d, Smem& sm, int bx, int by, int tile,
+                                        double& brate, double& lam, bool& bad, bool& nonq) {
   const Scalars* sc = d.sc;
   const int tid = threadIdx.y * TX + threadIdx.x;
   int tx, ty;
@@ -167,7 +167,6 @@ __device__ __forceinline__ void fv_tile(const Dev& d, Smem& sm, int bx, int by, 
   const double ts = STAGE == 1 ? sc->t : sc->t + dt;
   const double* __restrict__ In = STAGE == 1 ? d.S : d.T;
   const double g = d.g, tol = d.tol;
-  const int tile = by * d.tiles.ntx + bx;
   const bool every = !d.tiles.skip || d.tiles.all_forced || d.tiles.forced[tile];
   if (tid == 0) {
     const double k = STAGE == 1 ? dt : 0.5 * dt;
@@ -313,7 +312,7 @@ __device__ __forceinline__ void fv_tile(const Dev& d, Smem& sm, int bx, int by, 
 // only) writes the tiles' quiescence flags and the Courant rate; FV1's stage
 // leaves its result in T for fv1_commit_kernel.
 template <bool ORDER2, int STAGE>
-static __global__ void __launch_bounds__(TX* TY, 2) fv_stage_kernel(Dev d) {
+static __global__ void __launch_bounds__(TX* TY, 4) fv_stage_kernel(Dev d) {
   __shared__ Smem sm;
   Scalars* sc = d.sc;
   if (sc->done) return;
@@ -324,32 +323,33 @@ static __global__ void __launch_bounds__(TX* TY, 2) fv_stage_kernel(Dev d) {
   const bool all = sc->list_all != 0;
   double lam = 0.0;
   bool bad = false;
-  if (STAGE == 2 && (int)blockIdx.x >= n_act) return;
-  if ((int)blockIdx.x < n_act) {
-    const int tile = all ? (int)blockIdx.x : list_tile(d.tiles, sc, (int)blockIdx.x);
-    const int bx = tile % ntx, by = tile / ntx;
+  const int e = blockIdx.x / PARTS, part = blockIdx.x % PARTS;
+  if (STAGE == 2 && e >= n_act) return;
+  if (e < n_act) {
+    const int tile = all ? e : list_tile(d.tiles, sc, e);
+    const int tbx = tile % ntx, by = tile / ntx, bx = tbx * PARTS + part;
     double brate = 0.0;
     bool nonq = false;
-    fv_tile<ORDER2, STAGE>(d, sm, bx, by, brate, lam, bad, nonq);
-    if (bx == 0 || by == 0 || bx == ntx - 1 || by == d.tiles.nty - 1) {
+    if (bx * TX < d.nx) fv_tile<ORDER2, STAGE>(d, sm, bx, by, tile, brate, lam, bad, nonq);
+    if (tbx == 0 || by == 0 || tbx == ntx - 1 || by == d.tiles.nty - 1) {
       const double bsum = block_sum<TX * TY>(brate, sm.red);
       if (tx == 0 && ty == 0) {
-        d.bpart[(STAGE - 1) * d.tiles.ntiles + tile] = bsum;
+        d.bpart[((STAGE - 1) * d.tiles.ntiles + tile) * PARTS + part] = bsum;
         // FV1's one stage counts for both slots of the step's ledger average
-        if (!ORDER2) d.bpart[d.tiles.ntiles + tile] = bsum;
+        if (!ORDER2) d.bpart[(d.tiles.ntiles + tile) * PARTS + part] = bsum;
       }
     }
     if (last) {
       const int any_nonq = __syncthreads_or(nonq);
-      if (tx == 0 && ty == 0) d.tiles.flag[tile] = any_nonq ? 1 : 0;
+      if (tx == 0 && ty == 0) d.tiles.flag[tile * PARTS + part] = any_nonq ? 1 : 0;
     }
     __syncthreads();
   }
   if (STAGE == 1) {
-    const int e = (int)blockIdx.x - n_act;
-    if (e >= 0 && e < sc->n_front) {
-      const int tile = d.tiles.front[e];
-      const int i = (tile % ntx) * TX + tx, j = (tile / ntx) * TY + ty;
+    const int f = e - n_act;
+    if (f >= 0 && f < sc->n_front) {
+      const int tile = d.tiles.front[f];
+      const int i = (tile % ntx * PARTS + part) * TX + tx, j = (tile / ntx) * TY + ty;
       if (i < d.nx && j < d.ny) {
         const long long P = d.plane, c = (long long)j * d.pitch + i;
         d.T[H0 * P + c] = d.S[H0 * P + c];
@@ -369,11 +369,11 @@ static __global__ void __launch_bounds__(TX* TY, 2) fv_stage_kernel(Dev d) {
 static __global__ void __launch_bounds__(TX* TY) fv1_commit_kernel(Dev d) {
   const Scalars* sc = d.sc;
   if (sc->done) return;
-  const int n_act = sc->n_act;
-  if ((int)blockIdx.x >= n_act) return;
+  const int n_act = sc->n_act, e = blockIdx.x / PARTS, part = blockIdx.x % PARTS;
+  if (e >= n_act) return;
   const int ntx = d.tiles.ntx;
-  const int tile = sc->list_all ? (int)blockIdx.x : list_tile(d.tiles, sc, (int)blockIdx.x);
-  const int i = (tile % ntx) * TX + threadIdx.x, j = (tile / ntx) * TY + threadIdx.y;
+  const int tile = sc->list_all ? e : list_tile(d.tiles, sc, e);
+  const int i = (tile % ntx * PARTS + part) * TX + threadIdx.x, j = (tile / ntx) * TY + threadIdx.y;
   if (i >= d.nx || j >= d.ny) return;
   const long long P = d.plane, c = (long long)j * d.pitch + i;
   d.S[H0 * P + c] = d.T[H0 * P + c];
