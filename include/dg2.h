@@ -74,7 +74,8 @@ enum { DG2_WEST = 0, DG2_EAST = 1, DG2_SOUTH = 2, DG2_NORTH = 3 };
 typedef struct dg2_params {
     double g;           /* gravity, m/s^2 (default 9.80665)                         */
     double cfl;         /* Courant number Cr (Sec. 2.1.2; default 0.3)               */
-    double tol_dry;     /* drying tolerance on h (Sec. 2.1.3; default 1e-5 m)        */
+    double tol_dry;     /* drying tolerance on h (Sec. 2.1.3; default 1e-5 m); values
+                           below 1e-300 m act as 1e-300 m                            */
     double ds_thresh;   /* shock-detector threshold of Eq. 6 (default 10)            */
     double dt_max;      /* time step when no cell is wet, and upper cap (default 1 s)*/
     int variant;        /* DG2_NL or DG2_LL                                          */

@@ -1355,9 +1355,10 @@ __device__ __forceinline__ void stage_tile(const Dev& d, StageSmem<TX>& sm, int 
 // 44.8 ms, the 128 x 128 basin 13.5 -> 10.9 ms, with errors against an 80-bit run of the
 // same scheme 1.0 to 0.9 of what they were.
 //
-// 16 resident warps per SM are asked of the register allocator (128 registers a thread;
-// 2 blocks of 32 x 8 cells measured faster than 1 with 156 registers: DG2-LL floodplain
-// 0.857 against 0.955 ms per step).
+// 16 resident warps per SM are asked of the register allocator (128 registers a thread):
+// 4, 5 and 6 blocks of 16 x 8 cells took, stage 2 / stage 1 in us, 448 / 385, 437 / 375 and
+// 439 / 374 on the flooded plain, but 127 / 108, 129 / 112 and 133 / 113 on the DG2-NL
+// floodplain and 24.6 / 21.9, 25.3 / 22.4 and 26.5 / 23.2 on the 128 x 128 basin.
 // Stage kernels run over the step's list of active tiles (and, in stage 1,
 // the frontier tiles that only copy their state for a neighbour's halo),
 // built at the end of the previous step.
