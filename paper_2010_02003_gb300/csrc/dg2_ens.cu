@@ -573,7 +573,9 @@ int run_chunk(dg2_ens* e, int lv) {
 }
 
 // After the ensemble moved the members' states, their own tilings must
-// recompute every tile once.
+// recompute every tile once: their flags and lists still describe the states they
+// had before the call (dg2_set_state leaves exact ones), and water that has left
+// those tiles would stay frozen.
 int release_members(dg2_ens* e) {
   ECU(cudaStreamSynchronize(e->st));
   for (dg2_ctx* c : e->mem) {
@@ -582,6 +584,16 @@ int release_members(dg2_ens* e) {
     ECU(cudaStreamSynchronize(dg2::ctx_stream(c)));
   }
   return DG2_OK;
+}
+
+// The end of a call that may have stepped the members: releases them whatever the
+// call's result `r`, and returns r with its message (or the release's own failure).
+int release_after(dg2_ens* e, int r) {
+  if (!r) return release_members(e);
+  const std::string text = dg2_last_error();
+  release_members(e);
+  dg2::set_error_text(text.c_str());
+  return r;
 }
 
 int check_ens(dg2_ens* e) {
@@ -696,10 +708,11 @@ int dg2_ens_run_to(dg2_ens* e, double t_end, int64_t* steps_taken) {
   // Every live member advances its own t by a positive dt each step (a zero or
   // non-finite dt raises its non-finite flag), and lands on t_end exactly.
   while (s.n_done < n) {
-    if ((r = run_chunk(e, lv))) return r;
+    if ((r = run_chunk(e, lv))) return release_after(e, r);
     taken += kChunkMin << lv;
-    if ((r = read_es(e, &s))) return r;
-    if (s.bad) return efail(DG2_E_NONFINITE, "a member's state or step became non-finite");
+    if ((r = read_es(e, &s))) return release_after(e, r);
+    if (s.bad)
+      return release_after(e, efail(DG2_E_NONFINITE, "a member's state or step became non-finite"));
     if ((kChunkMin << lv) < kChunkMax) ++lv;
   }
   e->steps += taken;
@@ -750,13 +763,14 @@ int dg2_ens_autotune(dg2_ens* e, double t_end, int steps_per_trial, int* tile_w,
   }
   cudaEventDestroy(a);
   cudaEventDestroy(b);
-  if (r) return r;
+  if (r) return release_after(e, r);
   for (int k = 0; k < kNumShapes; ++k)
     if (e->tune_ms[k] < best) { best = e->tune_ms[k]; best_k = k; }
-  if ((r = set_shape(e, best_k))) return r;
+  if ((r = set_shape(e, best_k))) return release_after(e, r);
   EnsScalars s;
-  if ((r = read_es(e, &s))) return r;
-  if (s.bad) return efail(DG2_E_NONFINITE, "a member's state or step became non-finite");
+  if ((r = read_es(e, &s))) return release_after(e, r);
+  if (s.bad)
+    return release_after(e, efail(DG2_E_NONFINITE, "a member's state or step became non-finite"));
   if (tile_w) *tile_w = kShapes[best_k].w;
   if (tile_h) *tile_h = kShapes[best_k].h;
   return release_members(e);
