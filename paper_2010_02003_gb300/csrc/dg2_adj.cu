@@ -1193,7 +1193,8 @@ __global__ void __launch_bounds__(AX* AY, 4)
                      double Q, store* __restrict__ rev) {
   __shared__ FwdSmem sm;
   const int tid = threadIdx.x, tx = tid % AX, ty = tid / AX;
-  const int i0 = blockIdx.x * AX, j0 = blockIdx.y * AY, i = i0 + tx, j = j0 + ty;
+  const int ntx = (p.nx + AX - 1) / AX;  // blocks in rows of tiles (a grid's y has 65535 at most)
+  const int i0 = blockIdx.x % ntx * AX, j0 = blockIdx.x / ntx * AY, i = i0 + tx, j = j0 + ty;
   const bool act = i < p.nx && j < p.ny;
   const long long N = p.N, c = (long long)j * p.nx + i;
   const store* __restrict__ In = STAGE == 1 ? Us : U1;
@@ -1805,7 +1806,7 @@ int fwd_step(Ctx* a, int k, double t, const store* Uin, store* Uout, bool keep_r
 #ifdef DG2_ADJ_STORE32
   const unsigned tiles = blocks(a->lay.N), nt = 256;
 #else
-  const dim3 tiles((a->p.nx + AX - 1) / AX, (a->p.ny + AY - 1) / AY);
+  const unsigned tiles = (unsigned)((a->p.nx + AX - 1) / AX) * (unsigned)((a->p.ny + AY - 1) / AY);
   const unsigned nt = AX * AY;
 #endif
   fwd_friction_kernel<<<blocks(a->lay.N), 256, 0, a->st>>>(a->p, Uin, Us, dt);
