@@ -1173,12 +1173,17 @@ __global__ void __launch_bounds__(256) fwd_friction_kernel(Prob p, const store* 
 // tiles of AX x AY cells, one thread each, with the FP64 solver's records, faces and update
 // (dg2_device.cuh): every record is built and every face revised and fluxed once per tile.
 // The FP64 pipe bounds it.  One thread per cell without tiles built each record twice and
-// each face twice, with full divisions and roots: 434 / 442 us a launch at 512 x 512 cells
-// then, 146 / 161 us now (friction 146 -> 69 us).  16 x 8 rather than 32 x 8 cells: the calibration grids are small, and a tile's arithmetic is long
-// enough that whole SMs would idle in the last wave.  rev (may be null) takes the revised
-// depth and bed of each face (planes 2f, 2f + 1 of faces E, W, N, S), which the reverse
-// sweep's own-terms pass reads.
-constexpr int AX = 16, AY = 8;
+// each face twice, with divisions and library roots: 434 / 442 us a launch at 512 x 512
+// cells then, 146 / 161 us now (friction 146 -> 69 us).  Tiles are 16 x 8 rather than 32 x 8:
+// the calibration grids are small, and a tile's arithmetic is long enough that whole SMs
+// would idle in the last wave.  On grids one to three cells wide they are 1 x 128 or 2 x 64,
+// since 16 columns would leave most lanes without a cell: 12 forward steps of 1 x 262144 cells
+// 56.6 -> 6.1 ms (14.0 without tiles), of 2 x 131072 28.9 -> 5.6 (15.0); with 4 columns 16 x 8
+// takes 14.9 as the untiled form did.  rev (may be null) takes the revised depth and bed of
+// each face (planes 2f, 2f + 1 of faces E, W, N, S), which the reverse sweep's own-terms pass
+// reads.
+constexpr int kAdjTile = 128;  // cells of a tile
+template <int AX, int AY>
 struct FwdSmem {
   Rec e[AY][AX], n[AY][AX];              // east / north record of each cell
   Rec hw[AY], he[AY], hs[AX], hn[AX];    // records beyond the tile
@@ -1186,12 +1191,13 @@ struct FwdSmem {
   StageK k;
 };
 
-template <int STAGE>
-__global__ void __launch_bounds__(AX* AY, 4)
+template <int STAGE, int AX>
+__global__ void __launch_bounds__(kAdjTile, 4)
     fwd_stage_kernel(Prob p, const store* __restrict__ Us, const store* __restrict__ U1,
                      store* __restrict__ Uo, unsigned short* __restrict__ mask, double dt, double t,
                      double Q, store* __restrict__ rev) {
-  __shared__ FwdSmem sm;
+  constexpr int AY = kAdjTile / AX;
+  __shared__ FwdSmem<AX, AY> sm;
   const int tid = threadIdx.x, tx = tid % AX, ty = tid / AX;
   const int ntx = (p.nx + AX - 1) / AX;  // blocks in rows of tiles (a grid's y has 65535 at most)
   const int i0 = blockIdx.x % ntx * AX, j0 = blockIdx.x / ntx * AY, i = i0 + tx, j = j0 + ty;
@@ -1221,10 +1227,10 @@ __global__ void __launch_bounds__(AX* AY, 4)
   }
   // records beyond the tile: a neighbour's, or the ghost of the tile cell's own limit
   const int ni = p.nx - i0 < AX ? p.nx - i0 : AX, nj = p.ny - j0 < AY ? p.ny - j0 : AY;
-  {
-    const int kind = tid < AY ? 0 : tid < 2 * AY ? 1 : tid < 2 * AY + AX ? 2 : 3;
-    const int q = kind == 0 ? tid : kind == 1 ? tid - AY : kind == 2 ? tid - 2 * AY : tid - 2 * AY - AX;
-    if (tid < 2 * (AX + AY) && q < (kind <= 1 ? nj : ni)) {
+  for (int k = tid; k < 2 * (AX + AY); k += kAdjTile) {
+    const int kind = k < AY ? 0 : k < 2 * AY ? 1 : k < 2 * AY + AX ? 2 : 3;
+    const int q = kind == 0 ? k : kind == 1 ? k - AY : kind == 2 ? k - 2 * AY : k - 2 * AY - AX;
+    if (q < (kind <= 1 ? nj : ni)) {
       const int gi = i0 + (kind == 0 ? 0 : kind == 1 ? ni - 1 : q);
       const int gj = j0 + (kind <= 1 ? q : kind == 2 ? 0 : nj - 1);
       const int dir = kind <= 1 ? 1 : 2, side = kind & 1;
@@ -1266,9 +1272,9 @@ __global__ void __launch_bounds__(AX* AY, 4)
     sm.fy[ty][tx] = f;
     dpS = w.dp;
   }
-  {
-    const bool yf = tid >= AY;
-    const int q = yf ? tid - AY : tid;
+  for (int k = tid; k < AX + AY; k += kAdjTile) {
+    const bool yf = k >= AY;
+    const int q = yf ? k - AY : k;
     if (yf ? q < ni : q < nj) {
       FaceR f;
       Side b;
@@ -1804,18 +1810,22 @@ int fwd_step(Ctx* a, int k, double t, const store* Uin, store* Uout, bool keep_r
   unsigned short* m1 = (unsigned short*)(a->ws + a->lay.off_m1);
   unsigned short* m2 = (unsigned short*)(a->ws + a->lay.off_m2);
 #ifdef DG2_ADJ_STORE32
-  const unsigned tiles = blocks(a->lay.N), nt = 256;
+  const unsigned grid = blocks(a->lay.N), nt = 256;
+  auto *stage1 = fwd_stage_kernel<1>, *stage2 = fwd_stage_kernel<2>;
 #else
-  const unsigned tiles = (unsigned)((a->p.nx + AX - 1) / AX) * (unsigned)((a->p.ny + AY - 1) / AY);
-  const unsigned nt = AX * AY;
+  const int nx = a->p.nx, ax = nx == 1 ? 1 : nx < 4 ? 2 : 16, ay = kAdjTile / ax;
+  const unsigned grid = (unsigned)((nx + ax - 1) / ax) * (unsigned)((a->p.ny + ay - 1) / ay);
+  const unsigned nt = kAdjTile;
+  auto* stage1 = ax == 1 ? fwd_stage_kernel<1, 1> : ax == 2 ? fwd_stage_kernel<1, 2> : fwd_stage_kernel<1, 16>;
+  auto* stage2 = ax == 1 ? fwd_stage_kernel<2, 1> : ax == 2 ? fwd_stage_kernel<2, 2> : fwd_stage_kernel<2, 16>;
 #endif
   fwd_friction_kernel<<<blocks(a->lay.N), 256, 0, a->st>>>(a->p, Uin, Us, dt);
   store* rev = dptr(a, a->lay.off_rev);
   const long long r8 = 8 * (long long)a->lay.N;
-  fwd_stage_kernel<1><<<tiles, nt, 0, a->st>>>(a->p, Us, nullptr, U1, m1, dt, t, hydro(a, t),
-                                                    keep_rev ? rev : nullptr);
-  fwd_stage_kernel<2><<<tiles, nt, 0, a->st>>>(a->p, Us, U1, Uout, m2, dt, t + dt,
-                                                    hydro(a, t + dt), keep_rev ? rev + r8 : nullptr);
+  stage1<<<grid, nt, 0, a->st>>>(a->p, Us, nullptr, U1, m1, dt, t, hydro(a, t),
+                                 keep_rev ? rev : nullptr);
+  stage2<<<grid, nt, 0, a->st>>>(a->p, Us, U1, Uout, m2, dt, t + dt, hydro(a, t + dt),
+                                 keep_rev ? rev + r8 : nullptr);
   a->fwd_steps++;
   return launch_ok();
 }

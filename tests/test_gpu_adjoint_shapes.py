@@ -69,3 +69,36 @@ def compare(length, width, nsteps):
 
 def test_more_rows_of_tiles_than_a_launch_has_along_y():
     compare(8 * 65535 + 1, 1, 2)
+
+
+# widths either side of those at which the forward stage's tiles change, with lengths that end
+# inside a tile, at its end and one cell past it
+@pytest.mark.parametrize("length", [1, 63, 64, 65, 127, 128, 129, 300])
+@pytest.mark.parametrize("width", [1, 2, 3, 4, 5])
+def test_narrow_grids_give_the_transposed_result(length, width):
+    compare(length, width, 3)
+
+
+@pytest.mark.parametrize("width", [1, 2, 3])
+def test_a_narrow_grid_takes_no_longer_along_y(width):
+    """Least time of the forward steps of some 260 000 cells, along y and along x.  Tiles of
+    16 x 8 cells kept 1 to 3 of 16 lanes at work along y: 4.9, 4.5 and 3.1 times."""
+    import torch
+    from paper_2010_02003_gb300 import binding as B
+
+    length = 262144 // width
+    z, u, n = channel(length, width, 5)
+    best = []
+    for ydir in (False, True):
+        a, ws, _ = build(z, u, n, ydir, np.array([[0.5, 0.5]]), 8)
+        t = []
+        for _ in range(6):
+            e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            e0.record()
+            B.dg2_adj_forward(a, 1, 1)
+            e1.record()
+            torch.cuda.synchronize()
+            t.append(e0.elapsed_time(e1))
+        best.append(min(t[1:]))
+        B.dg2_adj_destroy(a)
+    assert best[1] <= 2.0 * best[0], best
