@@ -243,7 +243,8 @@ __device__ __forceinline__ double rcp64(double x) {
   e = fma(e, e, e);
   return fma(r, e, r);
 }
-// x >= 0; 0 below the normal range
+// 0 for arguments below the normal range (of either sign), else as sqrt: NaN for a negative
+// one and for a NaN
 __device__ __forceinline__ double sqrt64(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
@@ -252,7 +253,7 @@ __device__ __forceinline__ double sqrt64(double x) {
   const double t = x * y;
   double s = fma(fma(-t, t, x), h, t);
   s = fma(fma(-s, s, x), h, s);
-  return __double2hiint(x) < 0x00100000 ? 0.0 : s;
+  return (unsigned)__double2hiint(x) << 1 < 0x00200000u ? 0.0 : s;
 }
 // x / 2, on the integer units unless the result is below the normal range
 __device__ __forceinline__ double half64(double x) {
