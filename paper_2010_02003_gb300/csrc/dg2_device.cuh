@@ -1742,6 +1742,13 @@ static __global__ void __launch_bounds__(256) state_check_kernel(Dev d, unsigned
       return;
     }
 }
+// Whether a cell of the FV schemes has water that moves or may enter a neighbour.  Without
+// slopes (a dry cell has none) its deepest face depth is eta - (eta - h) (fv::face), which
+// rounding may put above tol_dry where h is not.
+__device__ __forceinline__ bool fv_moves(double eta, double h, double qx, double qy, double tol) {
+  return above(h, tol) || nonzero(qx) || nonzero(qy) ||
+         (is_pos(h) && above(eta - (eta - h), tol));
+}
 // One block per 32 x 8 tile.  The copy also writes the tiles' flags and the cell masks of the
 // new state, so the first step leaves still, dry ground out as every other does (computing
 // the whole grid there was a twentieth of a pass of 84 steps of a 2000 x 1000 floodplain).
@@ -1757,12 +1764,19 @@ static __global__ void __launch_bounds__(256) state_in_kernel(Dev d) {
   bool nq = false;
   if (i < d.nx && j < d.ny) {
     const long long n = (long long)d.nx * d.ny, c = (long long)j * d.nx + i;
+    const long long o = (long long)j * d.pitch + i;
+    double m[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-      const double v = d.T[k * n + c];
-      d.S[k * d.plane + (long long)j * d.pitch + i] = v;
-      if (k == 0) nq = above(v, d.tol) || v < -1.0;
-      else if (d.scheme == 0 || k % 3 == 0) nq = nq || nonzero(v);
+      m[k] = d.T[k * n + c];
+      d.S[k * d.plane + o] = m[k];
+    }
+    nq = above(m[H0], d.tol) || m[H0] < -1.0;
+    if (d.scheme != 0) {
+      nq = nq || fv_moves(m[H0] + d.Z[o], m[H0], m[QX0], m[QY0], d.tol);
+    } else {
+#pragma unroll
+      for (int k = 1; k < 9; ++k) nq = nq || nonzero(m[k]);
     }
   }
   const unsigned bits = __ballot_sync(0xffffffffu, nq);

@@ -545,8 +545,11 @@ static __global__ void __launch_bounds__(256) state_in32_kernel(D32 d, const dou
 }
 
 // The checked state from T to S, with the flags of the tiles (tw x 8 cells, 16 or 32 wide)
-// that hold a cell which is not still and dry, so the first step leaves the others out as
-// every step does.  One block per 32 x 8 cells.
+// that hold a cell which is not still and dry, so the first step leaves the others out.  A
+// film whose average is at most tol_dry may still have a face depth above it, by the rounding
+// of depths formed as eta - z, and then gives water to its neighbours: the test is of all
+// five depths, as the stage forms them, so that the first step is the one that computes every
+// tile.  One block per 32 x 8 cells.
 static __global__ void __launch_bounds__(256) state_commit32_kernel(D32 d, int tw) {
   __shared__ int moving[2];
   const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -564,9 +567,14 @@ static __global__ void __launch_bounds__(256) state_commit32_kernel(D32 d, int t
     }
     float z0, z1x, z1y, zE, zW, zN, zS;
     cell_z(d, i, j, z0, z1x, z1y, zE, zW, zN, zS);
-    nq = !((m[E0] - z0) + m[E0L] <= d.tol) || m[E1X] != z1x || m[E1Y] != z1y;
+    float eh, wh, nh, sh;
+    face_depths32(m[E0], m[E1X], m[E1Y], m[E0L], zE, zW, zN, zS, eh, wh, nh, sh);
+    nq = !((m[E0] - z0) + m[E0L] <= d.tol) || eh > d.tol || wh > d.tol || nh > d.tol || sh > d.tol;
+    // on the bits: a denormal, which the comparisons take for 0, is not still
+    nq = nq || __float_as_uint(m[E1X]) != __float_as_uint(z1x) ||
+         __float_as_uint(m[E1Y]) != __float_as_uint(z1y);
 #pragma unroll
-    for (int k = 3; k < 9; ++k) nq = nq || m[k] != 0.f;
+    for (int k = 3; k < 9; ++k) nq = nq || (__float_as_uint(m[k]) << 1) != 0;
   }
   if (nq) moving[threadIdx.x / tw] = 1;
   __syncthreads();

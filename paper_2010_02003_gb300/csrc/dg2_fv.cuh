@@ -17,7 +17,7 @@
 // carries over unchanged: a still, dry cell among still, dry neighbours has zero
 // fluxes, and the dry reset removes the discharge its bed term makes.  The same
 // holds for single cells, so a cell whose input and four neighbours are still and
-// dry (read off the staged averages) takes L = 0 and its faces are left out.
+// dry (read off the staged averages, fv_moves) takes L = 0 and its faces are left out.
 //
 // The FP64 pipe bounds the kernels.  Divisions (Sweby's ratio, the velocities) and FP64
 // comparisons used to make up most of their FP64 instructions, and every cell of a
@@ -196,7 +196,7 @@ __device__ __forceinline__ void fv_tile(const Dev& d, Smem& sm, int bx, int by, 
   bool b_me = act && every;
   if (act && !every) {
     auto moves = [&](int aa, int bb) {
-      return above(A[1][bb][aa], tol) || nonzero(A[2][bb][aa]) || nonzero(A[3][bb][aa]);
+      return fv_moves(A[0][bb][aa], A[1][bb][aa], A[2][bb][aa], A[3][bb][aa], tol);
     };
     b_me = moves(a, b) || moves(a - 1, b) || moves(a + 1, b) || moves(a, b - 1) || moves(a, b + 1);
   }
