@@ -86,7 +86,9 @@ typedef struct dg2_params {
     int skip_dry_tiles; /* 1 (default): leave 32 x 8 tiles of still, dry cells with
                            still, dry neighbours untouched -- they are exact fixed
                            points of a step, so results are bit-identical; 0: compute
-                           every tile */
+                           every tile.  (FP32 and the FV schemes form depths as eta - z:
+                           a film within rounding of tol_dry, dry by its average but
+                           not by a face depth, may lie still in such a tile.) */
     int flux;           /* Riemann solver: DG2_HLL (default) or DG2_ROE (Roe's solver
                            named in Sec. 2.1.2, Harten's entropy fix; DG2_FP64 only) */
     int scheme;         /* DG2_SCHEME_DG2 (default), or DG2_SCHEME_FV2 / DG2_SCHEME_FV1

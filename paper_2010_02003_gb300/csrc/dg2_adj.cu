@@ -924,8 +924,8 @@ __device__ __forceinline__ void friction_cell(const T* m, const T& n, real dt, r
 // Reverse-mode adjoint of one friction point (q /= 1 + gn2dt |q| h^(-7/3)): given the
 // adjoints (wx, wy) of the updated discharges, adds the gradient into g_gn2dt,
 // g_h, g_qx, g_qy (a dry point is the identity).  One reciprocal per denominator and
-// h^(-7/3) by its series: some 45 FP64 instructions, about 200 with a cube root and eight
-// divisions (adj_cell_kernel<1>, which is mostly this: 674 -> 180 us at 512 x 512).
+// h^(-7/3) by its series, in place of a cube root and eight divisions (adj_cell_kernel<1>,
+// which is mostly this: 674 -> 180 us at 512 x 512).
 __device__ __forceinline__ void friction_point_adj(real gn2dt, real tol, real h, real qx, real qy,
                                                    real wx, real wy, real& g_gn2dt, real& g_h,
                                                    real& g_qx, real& g_qy) {
@@ -1816,8 +1816,12 @@ int fwd_step(Ctx* a, int k, double t, const store* Uin, store* Uout, bool keep_r
   const int nx = a->p.nx, ax = nx == 1 ? 1 : nx < 4 ? 2 : 16, ay = kAdjTile / ax;
   const unsigned grid = (unsigned)((nx + ax - 1) / ax) * (unsigned)((a->p.ny + ay - 1) / ay);
   const unsigned nt = kAdjTile;
-  auto* stage1 = ax == 1 ? fwd_stage_kernel<1, 1> : ax == 2 ? fwd_stage_kernel<1, 2> : fwd_stage_kernel<1, 16>;
-  auto* stage2 = ax == 1 ? fwd_stage_kernel<2, 1> : ax == 2 ? fwd_stage_kernel<2, 2> : fwd_stage_kernel<2, 16>;
+  auto* stage1 = ax == 1   ? fwd_stage_kernel<1, 1>
+                 : ax == 2 ? fwd_stage_kernel<1, 2>
+                           : fwd_stage_kernel<1, 16>;
+  auto* stage2 = ax == 1   ? fwd_stage_kernel<2, 1>
+                 : ax == 2 ? fwd_stage_kernel<2, 2>
+                           : fwd_stage_kernel<2, 16>;
 #endif
   fwd_friction_kernel<<<blocks(a->lay.N), 256, 0, a->st>>>(a->p, Uin, Us, dt);
   store* rev = dptr(a, a->lay.off_rev);

@@ -54,11 +54,14 @@ size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 // Blocks per 32 x 8 tile of an FP64 context's lists.  The FP64 pipe takes a warp
 // instruction per 64 cycles from each of an SM's four schedulers, so a tile's 256 cells keep
 // an SM busy for 10 to 20 us a stage: finer blocks spread a short list over more SMs and
-// even out a long one, at the price of more records and faces on their edges.  Measured (us a step,
-// 32 -> 16 -> 8 columns a block; DG2-NL basins): 96^2 88.8, 64.5, 65.0; 128^2 88.7, 66.0,
-// 66.0; 256^2 143.6, 143.9, 135.6; 384^2 259.9, 257.0, 266.7; 1024^2 1618, 1607, 1658;
-// floodplains 500 x 300 136, 124, 107; 1237 x 731 317, 299, 308; 2000 x 1000 (DG2-LL) 259,
-// 250, 265.  So 16 columns, and 8 on grids of up to two tiles per SM.
+// even out a long one, at the price of more records and faces on their edges.  Measured (us
+// a step, 32, 16, 8 columns a block; * the rule's choice; DG2-NL basins): 96^2 88.8, 64.5,
+// 65.0*; 128^2 88.7, 66.0, 66.0*; 256^2 143.6, 143.9, 135.6*; 384^2 259.9, 257.0*, 266.7;
+// 1024^2 1618, 1607*, 1658; floodplains 500 x 300 136, 124*, 107; 1237 x 731 317, 299*, 308;
+// 2000 x 1000 (DG2-LL) 259, 250*, 265.  What counts is the listed tiles; the layout of the
+// workspace needs the width before there are any, so the line is at twice 152 tiles (two a
+// SM) of the grid, and a partly wet grid a little above it, as 500 x 300, gets 16 columns
+// where 8 would be faster.
 constexpr int kFineTiles = 304;
 int parts64(int nx, int ny, int scheme) {
   if (scheme != DG2_SCHEME_DG2) return dg2::fv::PARTS;
@@ -323,7 +326,7 @@ void enqueue_step(dg2_ctx* c, bool timed = false) {
   }
   if (e) cudaEventRecord(e[1], c->st);
   if (c->p.scheme != DG2_SCHEME_DG2) {
-    // the FV comparators: one block per tile of the lists, as the DG2 stages
+    // the FV comparators: one block per half tile of the lists, as the DG2 stages
     if (c->p.scheme == DG2_SCHEME_FV2)
       dg2::fv::fv_stage_kernel<true, 1><<<c->g_st1, c->sblock, 0, c->st>>>(d);
     else
@@ -385,8 +388,8 @@ void launch_mass(dg2_ctx* c) {
   else dg2::mass_kernel<<<c->pgrid, c->pblock, 0, c->st>>>(c->d);
 }
 
-// Marks every tile non-quiescent so the next step computes the whole grid
-// (after a new DEM or state; the first stage 2 then sets the true flags).
+// Marks every tile non-quiescent so the next step computes the whole grid (after a new
+// DEM, or when an ensemble moved the state; the first stage 2 then sets the true flags).
 int reset_tiles(dg2_ctx* c) {
   CU(cudaMemsetAsync(c->d.tiles.flag, 1, (size_t)c->lay.nblocks * c->d.nsub, c->st));
   // every cell non-quiescent in the cell masks: the first step computes every cell
@@ -409,8 +412,8 @@ int reset_ledger(dg2_ctx* c) {
 
 namespace {
 
-// FP32 contexts: host copies of the face topography and the cell modes of z
-// formed exactly as the kernels form them (FP32 sums of face values).
+// FP32 contexts, for dg2_get_topo: the cell modes of z from host copies of the face
+// topography, formed exactly as the kernels form them (FP32 sums of face values).
 int f32_topo_modes(dg2_ctx* c, std::vector<float>& z0, std::vector<float>& z1x,
                    std::vector<float>& z1y) {
   const int nx = c->f.nx, ny = c->f.ny;
@@ -594,21 +597,14 @@ int dg2_init_grid(dg2_ctx** out, int nx, int ny, double dx, double dy, const dg2
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     const bool ll = p.variant == DG2_LL, f32 = p.precision == DG2_FP32;
     int o1 = 1, o2 = 1;
-    // the FP64 stage tile's shared memory is above the 48 KB static limit
-    if (!f32)
-      for (int stage = 1; stage <= 2 && p.scheme == DG2_SCHEME_DG2; ++stage)
-        cudaFuncSetAttribute(stage64(c, stage), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)stage64_smem(c));
-    if (f32) {
-      dg2::ens::occupancy32(tile_w(c), ll, &o1, &o2);
-    }
+    if (f32) dg2::ens::occupancy32(tile_w(c), ll, &o1, &o2);
     cudaGetLastError();
     const int nt = d.tiles.ntiles;
     auto gsz = [&](int occ) { long long g = (long long)nsm * (occ > 0 ? occ : 1); return (int)(g < nt ? g : nt); };
     c->lblock = dim3(dg2::LTX, dg2::LTY);
     c->lgrid = dim3((d.tiles.ntx + dg2::LTX - 1) / dg2::LTX, (d.tiles.nty + dg2::LTY - 1) / dg2::LTY);
-    // friction: one block per tile of the list (the hardware hands blocks to SMs
-    // as they free up); measured faster than a persistent grid looping over the
+    // friction: one block per part of a tile of the list (the hardware hands blocks to
+    // SMs as they free up); measured faster than a persistent grid looping over the
     // list (floodplain 2000 x 1000 from t = 1 h: 0.060 -> 0.051 ms per step)
     c->g_fric = nt * d.nsub;
     c->g_st1 = f32 ? gsz(o1) : nt * d.nsub;

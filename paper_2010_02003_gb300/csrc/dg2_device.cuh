@@ -1,18 +1,20 @@
 // dg2_device.cuh -- device code of the GB300 DG2 solver (sm_103a).
 //
 // One RK2 step of the slope-decoupled DG2 scheme (Sec. 2.1 of Ayog et al.)
-// is three launches on the caller's stream:
+// is four or five launches on the caller's stream:
 //   friction_kernel   implicit Manning friction at the centre and the four
 //                     Gauss points of every cell (Sec. 2.1.3), in place;
 //   stage_kernel<1>   [local limiting, Eqs. 6-7] + spatial operator
 //                     (Eqs. 4-5) + U1 = Un + dt L(Un) + wet-dry treatment;
 //   stage_kernel<2>   [limiting] + operator + Un+1 = (Un + U1 + dt L(U1)) / 2
 //                     + wet-dry treatment, then the Courant-number reduction
-//                     for the next step; its last block to finish advances t,
-//                     the mass ledger and the gauges (no host round trip).
+//                     for the next step;
+//   finalize_kernel   t, the mass ledger, the gauges and the next step's size, and
+//   lists_kernel      the next step's tile lists (grids of up to kSmallTiles tiles:
+//                     both in finalize_small_kernel).  No host round trip.
 //
 // Layout: structure of arrays, one FP64 plane per coefficient, row pitch a
-// multiple of 32 elements.  A block owns a TX x TY tile of cells; it computes
+// multiple of 32 elements.  A block owns a TX x TY part of a tile; it computes
 // every revised face limit once (Sec. 2.1.2), keeps the east/north limits in
 // shared memory so each interior face flux is evaluated once per tile, and
 // evaluates the halo limits (and ghost states on domain edges) itself.
@@ -228,14 +230,13 @@ __device__ __forceinline__ bool nonzero(double x) { return (fbits(x) << 1) != 0;
 // ---------------------------------------------------------------------------
 // FP64 reciprocal and square root in few FP64 instructions
 // ---------------------------------------------------------------------------
-// The FP64 pipe bounds the stage kernels, and a compiled 1 / x or sqrt(x) is about
-// nine instructions on it with a branch to a slow path.  These start from the
-// hardware's 32-bit-mantissa-word approximations (PTX rcp.approx / rsqrt.approx)
-// and refine them: the reciprocal by one third-order Householder step
-// r (1 + e + e^2), e = 1 - x r (3 instructions); the root by two of Heron's steps
-// s + (x - s^2) y / 2 with the same y ~ x^(-1/2) (5 instructions), whose residuals
-// are exact to a rounding.  Over 2^28 arguments the relative residuals stay below
-// 1.01 x 2^-53 (the approximations': 1.0e-6 and 1.9e-6).
+// The FP64 pipe bounds the stage kernels.  These start from PTX's approximations
+// (rcp.approx / rsqrt.approx, errors up to 1.0e-6 and 1.9e-6) and refine them: the
+// reciprocal by one third-order Householder step r (1 + e + e^2), e = 1 - x r (3
+// instructions); the root by two of Heron's steps s + (x - s^2) y / 2 with the same
+// y ~ x^(-1/2) (5 instructions), whose residuals are exact to a rounding.  That leaves
+// relative errors of at most 1.01 x 2^-53 and 1.1 x 2^-53
+// (tests/fp64_helpers_check.cu).  For normal arguments whose reciprocal is normal.
 __device__ __forceinline__ double rcp64(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
@@ -682,7 +683,8 @@ static __global__ void init_kernel(Dev d, const double* __restrict__ zc, const d
 // For h in (1e-30, 1e30), h^(-7/3) comes from the FP32 inverse cube root r of h (cut to
 // FP32 on the integer units) and the binomial series about it: h = (1 - e) / r^3 with
 // |e| < 1e-6, so h^(-7/3) = r^7 (1 + 7/3 e + 35/9 e^2 + O(6 e^3)), 8 FP64 instructions and
-// no conversion; two Newton steps on the root took about 20.  Outside, h^2 cbrt(h) divides.
+// no conversion, within 3.7 x 2^-53; two Newton steps on the root took about 20.  Outside,
+// 1 / (h^2 cbrt(h)).
 __device__ __forceinline__ double h_m73(double h) {
   if (!(fbits(h) > fbits(1e-30) && fbits(h) < fbits(1e30))) return 1.0 / (h * h * cbrt(h));
   const float hf = __int_as_float(((__double2hiint(h) - 0x38000000) << 3) |
@@ -1342,19 +1344,20 @@ __device__ __forceinline__ void stage_tile(const Dev& d, StageSmem<TX>& sm, int 
   }
 }
 
-// Work distribution of the stage kernels over the step's tile lists: one block per tile
-// of the grid, and a block takes the entry of its own index (blocks past the lists exit
-// at once, and the hardware balances tiles of unequal cost over the SMs).  On the
-// 2000 x 1000 floodplain FP64 tiles (tens of microseconds each, 1-2 blocks per SM) run
-// faster so than in resident blocks that loop over the list; the FP32 kernels (shared
-// with ensembles) loop.
+// Work distribution of the stage kernels over the step's tile lists: one block per part of
+// a tile of the grid, and a block takes the part of its own index of the list (blocks past
+// the lists exit at once, and the hardware balances tiles of unequal cost over the SMs).  On
+// the 2000 x 1000 floodplain FP64 tiles ran faster so than in resident blocks that loop over
+// the list; the FP32 kernels (shared with ensembles) loop.
 // The FP64 pipe bounds both stages (two lanes an SM and cycle against 128 FP32 ones).
 // Their arithmetic in fewer FP64 instructions (rcp64 / sqrt64, hll, the deviation form of
 // Flux, folded step weights, friction's series) took whole passes from the start of this
 // form to its end (state in, run, state out): 2000 x 1000 floodplain DG2-LL 42.7 -> 29.9 ms,
 // 1237 x 731 floodplain DG2-NL 36.8 -> 27.1 ms, 1000 x 600 flooded plain DG2-LL 58.5 ->
-// 44.8 ms, the 128 x 128 basin 13.5 -> 10.9 ms, with errors against an 80-bit run of the
-// same scheme 1.0 to 0.9 of what they were.
+// 44.8 ms, the 128 x 128 basin 13.5 -> 10.9 ms.  Errors against a plain 64-bit statement of
+// the scheme, geometric mean of the ratios to the form before over 12 inputs each: 0.95, 1.02,
+// 0.94 and 0.95 in that order, FV2 floodplain 1.01 (single inputs beside banks 0.5 to 2.7,
+// where one cell's round-off grows).
 //
 // 16 resident warps per SM are asked of the register allocator (128 registers a thread):
 // 4, 5 and 6 blocks of 16 x 8 cells took, stage 2 / stage 1 in us, 448 / 385, 437 / 375 and
@@ -1366,7 +1369,8 @@ __device__ __forceinline__ void stage_tile(const Dev& d, StageSmem<TX>& sm, int 
 template <bool LL, int STAGE, bool ROE, int TX>
 static __global__ void __launch_bounds__(TX* TY, 2 * TW / TX) stage_kernel(Dev d) {
   constexpr int TBX = TX / WX, PARTS = TW / TX;
-  extern __shared__ double stage_smem[];  // one StageSmem (dynamic: may pass 48 KB)
+  extern __shared__ double stage_smem[];  // one StageSmem
+  static_assert(sizeof(StageSmem<TX>) <= 48 * 1024, "the default limit of dynamic shared memory");
   StageSmem<TX>& sm = *reinterpret_cast<StageSmem<TX>*>(stage_smem);
   Scalars* sc = d.sc;
   if (sc->done) return;
